@@ -62,54 +62,152 @@ void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, dim3 grid
 }
 
 // ---------------------------------------------------------------------------------------
-// Window statistics (Sec. IV-B-1, Eq. (sum1), Method 1 made separable): block per row y;
-// column sums of the 2r+1 clamped rows for every column the row's windows touch, then the
-// horizontal window sum of those. S, Q exact int32; inv_sigma = rsqrtf(n Q - S^2) (within 2
+// Window statistics (Sec. IV-B-1, Eq. (sum1), Method 1 made separable). A block covers
+// kStatsCols image columns, four adjacent ones per thread, and walks kStatsRows rows down:
+// a thread keeps its columns' sums over the 2r+1 clamped rows and, from row to row, adds the
+// row that enters and subtracts the one that leaves (exact in int32), so that a pixel is read
+// about (2r+1)/kStatsRows + 2 times instead of 2r+1 times, four at a time where the rows are
+// 4-byte aligned. The row's column sums go through shared memory (two buffers, one barrier a
+// row) and each thread sums the windows of four adjacent centres from 16-byte reads.
+// Bound by latency and launch at these sizes (26 MB in all at 1920x1080); one block per row
+// with a byte load per pixel and window row took 25.0 us there, this 10.4.
+// S, Q exact int32; inv_sigma = rsqrtf(n Q - S^2) (within 2
 // ulp of 1/sqrt) or 0; the cost kernel computes its statistics the same way, bit for bit.
 // n Q - S^2 < 2^31 for every window side <= 15 (its maximum is n^2 * 127.5^2), so it is
 // computed modulo 2^32 in unsigned arithmetic even where n Q alone would not fit.
 // `packed` receives (S, inv_sigma bits) per centre for the cost kernel.
-__global__ void k_window_stats(const uint8_t* __restrict__ img, int pitch, int W, int H, int r,
-                               int x_begin, int nx, int* __restrict__ S, int* __restrict__ Q,
-                               float* __restrict__ isig, int2* __restrict__ packed) {
-    extern __shared__ int sm_stats[];
-    const int y = blockIdx.x;
-    const int ncol = nx + 2 * r;
-    int* cs = sm_stats;
-    int* cq = sm_stats + ncol;
-    for (int t = threadIdx.x; t < ncol; t += blockDim.x) {
-        const int xc = min(max(x_begin - r + t, 0), W - 1);
-        int s = 0, q = 0;
-        for (int j = -r; j <= r; ++j) {
-            const int p = img[(size_t)min(max(y + j, 0), H - 1) * pitch + xc];
-            s += p;
-            q += p * p;
-        }
-        cs[t] = s;
-        cq[t] = q;
+constexpr int kStatsThreads = 128;
+constexpr int kStatsCols = 4 * kStatsThreads;
+constexpr int kStatsRows = 8;
+// Centres per block: its columns less the windows' reach and up to three columns that align
+// its first column to four image columns.
+constexpr int stats_centres(int r) { return (kStatsCols - 2 * r - 3) & ~3; }
+
+template <int R>
+__global__ void __launch_bounds__(kStatsThreads)
+k_window_stats(const uint8_t* __restrict__ img, int pitch, int W, int H, int x_begin, int nx, int words,
+               int vec, int* __restrict__ S, int* __restrict__ Q, float* __restrict__ isig,
+               int2* __restrict__ packed) {
+    constexpr int OUT = stats_centres(R);
+    constexpr int NV = (4 + 2 * R + 3) / 4;              // 16-byte reads that cover four windows
+    __shared__ __align__(16) int cs[2][kStatsCols + 4 * NV], cq[2][kStatsCols + 4 * NV];
+    const int i = threadIdx.x;
+    const int o0 = blockIdx.x * OUT, y0 = blockIdx.y * kStatsRows;
+    const int sh = (x_begin - R + o0) & 3;               // columns before the first window's
+    const int xa = x_begin - R + o0 - sh + 4 * i;        // this thread's columns xa .. xa + 3
+    const bool word = words && xa >= 0 && xa + 3 < W;    // (xa is a multiple of 4)
+    int xc[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) xc[c] = min(max(xa + c, 0), W - 1);
+    auto row = [&](int y) -> unsigned {                  // the four pixels of a clamped row
+        const uint8_t* p = img + (size_t)min(max(y, 0), H - 1) * pitch;
+        if (word) return *reinterpret_cast<const unsigned*>(p + xa);
+        return (unsigned)p[xc[0]] | (unsigned)p[xc[1]] << 8 | (unsigned)p[xc[2]] << 16 | (unsigned)p[xc[3]] << 24;
+    };
+    int s[4] = {0, 0, 0, 0}, q[4] = {0, 0, 0, 0};
+    {
+        unsigned w[2 * R + 1];
+#pragma unroll
+        for (int j = 0; j <= 2 * R; ++j) w[j] = row(y0 - R + j);
+#pragma unroll
+        for (int j = 0; j <= 2 * R; ++j)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int v = (int)(w[j] >> (8 * c) & 255u);
+                s[c] += v;
+                q[c] += v * v;
+            }
     }
-    __syncthreads();
-    const unsigned n = (unsigned)((2 * r + 1) * (2 * r + 1));
-    for (int t = threadIdx.x; t < nx; t += blockDim.x) {
-        int s = 0, q = 0;
-        for (int i = 0; i <= 2 * r; ++i) {
-            s += cs[t + i];
-            q += cq[t + i];
+    const unsigned n = (unsigned)((2 * R + 1) * (2 * R + 1));
+    const int y1 = min(y0 + kStatsRows, H), o = o0 + 4 * i;
+    for (int y = y0; y < y1; ++y) {
+        const unsigned in = row(y + 1 + R), out = row(y - R);       // (used after this row)
+        int* bs = cs[y & 1];
+        int* bq = cq[y & 1];
+        if (sh == 0) {
+            *reinterpret_cast<int4*>(bs + 4 * i) = make_int4(s[0], s[1], s[2], s[3]);
+            *reinterpret_cast<int4*>(bq + 4 * i) = make_int4(q[0], q[1], q[2], q[3]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (4 * i + c >= sh) {
+                    bs[4 * i + c - sh] = s[c];
+                    bq[4 * i + c - sh] = q[c];
+                }
         }
-        const size_t o = (size_t)y * nx + t;
-        const int var = (int)(n * (unsigned)q - (unsigned)s * (unsigned)s);
-        const float is = var > 0 ? rsqrtf((float)var) : 0.0f;
-        if (S) S[o] = s;
-        if (Q) Q[o] = q;
-        if (isig) isig[o] = is;
-        if (packed) packed[o] = make_int2(s, __float_as_int(is));
+        __syncthreads();
+        if (4 * i < OUT && o < nx) {
+            int a[4 * NV], b[4 * NV];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                const int4 u = *reinterpret_cast<const int4*>(bs + 4 * i + 4 * k);
+                const int4 v = *reinterpret_cast<const int4*>(bq + 4 * i + 4 * k);
+                a[4 * k] = u.x; a[4 * k + 1] = u.y; a[4 * k + 2] = u.z; a[4 * k + 3] = u.w;
+                b[4 * k] = v.x; b[4 * k + 1] = v.y; b[4 * k + 2] = v.z; b[4 * k + 3] = v.w;
+            }
+            int ws[4], wq[4];
+            float is[4];
+            ws[0] = wq[0] = 0;
+#pragma unroll
+            for (int k = 0; k <= 2 * R; ++k) {
+                ws[0] += a[k];
+                wq[0] += b[k];
+            }
+#pragma unroll
+            for (int c = 1; c < 4; ++c) {
+                ws[c] = ws[c - 1] + a[2 * R + c] - a[c - 1];
+                wq[c] = wq[c - 1] + b[2 * R + c] - b[c - 1];
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int var = (int)(n * (unsigned)wq[c] - (unsigned)ws[c] * (unsigned)ws[c]);
+                is[c] = var > 0 ? rsqrtf((float)var) : 0.0f;
+            }
+            const size_t at = (size_t)y * nx + o;
+            if (vec && o + 3 < nx) {
+                if (S) *reinterpret_cast<int4*>(S + at) = make_int4(ws[0], ws[1], ws[2], ws[3]);
+                if (Q) *reinterpret_cast<int4*>(Q + at) = make_int4(wq[0], wq[1], wq[2], wq[3]);
+                if (isig) *reinterpret_cast<float4*>(isig + at) = make_float4(is[0], is[1], is[2], is[3]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (o + c < nx) {
+                        if (S) S[at + c] = ws[c];
+                        if (Q) Q[at + c] = wq[c];
+                        if (isig) isig[at + c] = is[c];
+                    }
+            }
+            if (packed)
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (o + c < nx) packed[at + c] = make_int2(ws[c], __float_as_int(is[c]));
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int v = (int)(in >> (8 * c) & 255u), u = (int)(out >> (8 * c) & 255u);
+            s[c] += v - u;
+            q[c] += v * v - u * u;
+        }
     }
 }
 
 cudaError_t launch_window_stats(const uint8_t* img, int pitch, int W, int H, int r, int x_begin,
                                 int nx, int* S, int* Q, float* isig, int2* packed, cudaStream_t st) {
-    const size_t smem = 2 * sizeof(int) * (size_t)(nx + 2 * r);
-    k_window_stats<<<H, 256, smem, st>>>(img, pitch, W, H, r, x_begin, nx, S, Q, isig, packed);
+    const dim3 grid((nx + stats_centres(r) - 1) / stats_centres(r), (H + kStatsRows - 1) / kStatsRows);
+    // four pixels a load where the rows start on 4 bytes; four results a store where every
+    // output row starts on 16
+    const int words = (uintptr_t)img % 4 == 0 && pitch % 4 == 0;
+    const int vec = nx % 4 == 0 && (uintptr_t)S % 16 == 0 && (uintptr_t)Q % 16 == 0 && (uintptr_t)isig % 16 == 0;
+#define ZNCC_STATS(R)                                                                                        \
+    case R:                                                                                                  \
+        k_window_stats<R><<<grid, kStatsThreads, 0, st>>>(img, pitch, W, H, x_begin, nx, words, vec, S, Q, isig, \
+                                                          packed);                                           \
+        break;
+    switch (r) {
+        ZNCC_STATS(1) ZNCC_STATS(2) ZNCC_STATS(3) ZNCC_STATS(4) ZNCC_STATS(5) ZNCC_STATS(6) ZNCC_STATS(7)
+        default: return cudaErrorInvalidValue;
+    }
+#undef ZNCC_STATS
     return cudaGetLastError();
 }
 

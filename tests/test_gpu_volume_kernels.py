@@ -1,0 +1,39 @@
+"""Window statistics and WTA of a stored volume at the edges of their kernels' tiles, alignments
+and loads: whole numbers, compared exactly (1/sigma to its float rounding)."""
+
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2212_00476_gb300 import zncc as Z  # noqa: E402
+
+
+# (W, H, r, bytes from an aligned address to the first pixel, pitch - W): widths around the
+# centres of a block (512 columns less the window), heights around its 8 rows, rows that do and
+# do not start on 4 bytes
+@pytest.mark.parametrize("w,h,r,off,pad", [
+    (506, 8, 1, 0, 2), (507, 9, 1, 0, 1), (508, 7, 1, 4, 0), (1000, 17, 4, 0, 0), (1001, 16, 4, 1, 3),
+    (499, 3, 5, 2, 1), (500, 24, 5, 0, 4), (494, 8, 7, 0, 2), (495, 1, 7, 0, 1), (3, 40, 7, 3, 2), (1, 1, 2, 0, 0)])
+def test_window_stats_tiles_and_alignment(w, h, r, off, pad):
+    rng = np.random.default_rng(w + 31 * h + r)
+    pitch = w + pad
+    buf = rng.integers(0, 256, off + pitch * h + 64, dtype=np.uint8)
+    dev = torch.from_numpy(buf).cuda()
+    img = dev[off:off + pitch * h].view(h, pitch)[:, :w]
+    with Z.ZnccContext(w, h, 4, 2 * r + 1) as ctx:
+        S, Q = (torch.empty((h, w), dtype=torch.int32, device="cuda") for _ in range(2))
+        inv = torch.empty((h, w), dtype=torch.float32, device="cuda")
+        ctx.zncc_window_stats(img, S, Q, inv)
+        S2 = torch.zeros(h * w + 1, dtype=torch.int32, device="cuda")       # rows off 16 bytes
+        assert Z.lib().zncc_window_stats(ctx._h, img.data_ptr(), pitch, S2[1:].data_ptr(), None, None) == Z.ZNCC_OK
+        torch.cuda.synchronize()
+    s, q = oracle.window_sums(np.ascontiguousarray(img.cpu().numpy()), r)
+    assert np.array_equal(S.cpu().numpy(), s) and np.array_equal(Q.cpu().numpy(), q)
+    assert np.array_equal(S2[1:].view(h, w).cpu().numpy(), s)
+    var = (2 * r + 1) ** 2 * q.astype(np.int64) - s.astype(np.int64) ** 2
+    ref = np.where(var > 0, 1.0 / np.sqrt(np.maximum(var, 1)), 0.0)
+    assert np.allclose(inv.cpu().numpy(), ref, rtol=4e-7, atol=0)
