@@ -965,34 +965,82 @@ cudaError_t launch_wta_finish(const WtaFinishBatch& b, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------------------
-// WTA over a stored volume (Sec. III-C, Eq. (WTA1)): one warp per pixel, the smallest d
-// among the largest costs.
-template <typename T>
-__global__ void k_wta_volume(const T* __restrict__ cost, int npix, int D, uint16_t* __restrict__ disp) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= npix) return;
-    const T* c = cost + (size_t)warp * D;
+// WTA over a stored volume (Sec. III-C, Eq. (WTA1)): the smallest d among the largest costs.
+// Bound by reading the volume once. LP consecutive lanes share a pixel and each reads VEC
+// entries at a time (16 bytes where the pixels are aligned), so that a warp's loads are whole
+// 128-byte lines and kWtaLoads of them are in flight per lane; the warp-per-pixel kernel this
+// replaces had one 4-byte load per lane in flight and five shuffle rounds per pixel
+// (1280x384x128 F32: 67.6 -> 39.2 us, 6.4 TB/s).
+constexpr int kWtaLoads = 4;
+
+template <typename T, int VEC, int LP>
+__global__ void __launch_bounds__(256) k_wta_volume(const T* __restrict__ cost, int npix, int D,
+                                                    uint16_t* __restrict__ disp) {
+    const int lane = threadIdx.x & 31, sub = lane & (LP - 1);
+    const long long pix = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / LP;
+    const T* c = cost + (size_t)min(pix, (long long)npix - 1) * D;
     float best = -INFINITY;
     int bd = 0x7FFFFFFF;
-    for (int d = lane; d < D; d += 32) {
-        const float v = (float)c[d];
-        if (v > best) { best = v; bd = d; }
+    struct alignas(VEC * sizeof(T)) Vec { T v[VEC]; };
+    for (int d0 = sub * VEC; d0 < D; d0 += LP * VEC * kWtaLoads) {
+        Vec t[kWtaLoads];
+#pragma unroll
+        for (int k = 0; k < kWtaLoads; ++k)
+            if (d0 + k * LP * VEC < D) t[k] = *reinterpret_cast<const Vec*>(c + d0 + k * LP * VEC);
+#pragma unroll
+        for (int k = 0; k < kWtaLoads; ++k) {
+            const int d = d0 + k * LP * VEC;
+            if (d < D)                              // (VEC divides D: whole vectors)
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) {
+                    const float v = (float)t[k].v[j];
+                    if (v > best) { best = v; bd = d + j; }
+                }
+        }
     }
-    for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+    for (int off = LP / 2; off > 0; off >>= 1) {
         const float ob = __shfl_xor_sync(kFull, best, off);
         const int od = __shfl_xor_sync(kFull, bd, off);
         if (ob > best || (ob == best && od < bd)) { best = ob; bd = od; }
     }
-    if (lane == 0) disp[warp] = (uint16_t)(bd == 0x7FFFFFFF ? 0 : bd);
+    if (sub == 0 && pix < npix) disp[pix] = (uint16_t)(bd == 0x7FFFFFFF ? 0 : bd);
 }
 
+// Lanes per pixel: enough that each lane has about kWtaLoads loads, so that the shuffle rounds
+// serve many entries and no load slot stays empty.
+template <typename T, int VEC>
+static void wta_volume(const T* cost, int npix, int D, uint16_t* disp, cudaStream_t st) {
+    const int loads = D / VEC;
+    const int lp = loads <= 2 * kWtaLoads ? 2 : loads <= 4 * kWtaLoads ? 4 : loads <= 8 * kWtaLoads ? 8
+                   : loads <= 16 * kWtaLoads ? 16 : 32;
+    const int blocks = (int)(((long long)npix * lp + 255) / 256);
+    switch (lp) {
+        case 2: k_wta_volume<T, VEC, 2><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
+        case 4: k_wta_volume<T, VEC, 4><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
+        case 8: k_wta_volume<T, VEC, 8><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
+        case 16: k_wta_volume<T, VEC, 16><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
+        default: k_wta_volume<T, VEC, 32><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
+    }
+}
+
+// The widest load that every pixel's entries allow (base address and D): 16 or 8 bytes, else
+// one entry at a time.
 cudaError_t launch_wta_volume(const void* cost, int dtype, int W, int H, int D, uint16_t* disp,
                               cudaStream_t st) {
     const int npix = W * H;
-    const int blocks = (npix + 7) / 8;
-    if (dtype == 0) k_wta_volume<float><<<blocks, 256, 0, st>>>((const float*)cost, npix, D, disp);
-    else k_wta_volume<__half><<<blocks, 256, 0, st>>>((const __half*)cost, npix, D, disp);
+    const uintptr_t p = (uintptr_t)cost;
+    if (dtype == 0) {
+        const float* c = (const float*)cost;
+        if (D % 4 == 0 && p % 16 == 0) wta_volume<float, 4>(c, npix, D, disp, st);
+        else if (D % 2 == 0 && p % 8 == 0) wta_volume<float, 2>(c, npix, D, disp, st);
+        else wta_volume<float, 1>(c, npix, D, disp, st);
+    } else {
+        const __half* c = (const __half*)cost;
+        if (D % 8 == 0 && p % 16 == 0) wta_volume<__half, 8>(c, npix, D, disp, st);
+        else if (D % 4 == 0 && p % 8 == 0) wta_volume<__half, 4>(c, npix, D, disp, st);
+        else wta_volume<__half, 1>(c, npix, D, disp, st);
+    }
     return cudaGetLastError();
 }
 

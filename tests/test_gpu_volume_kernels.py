@@ -37,3 +37,29 @@ def test_window_stats_tiles_and_alignment(w, h, r, off, pad):
     var = (2 * r + 1) ** 2 * q.astype(np.int64) - s.astype(np.int64) ** 2
     ref = np.where(var > 0, 1.0 / np.sqrt(np.maximum(var, 1)), 0.0)
     assert np.allclose(inv.cpu().numpy(), ref, rtol=4e-7, atol=0)
+
+
+# D around the lanes per pixel and loads per lane, volumes that start off 16 bytes
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("d,off", [(1, 0), (2, 0), (3, 1), (8, 0), (8, 1), (31, 0), (32, 0), (33, 0), (36, 2),
+                                   (64, 0), (66, 0), (128, 0), (132, 4), (256, 0), (260, 0), (1021, 0), (1024, 0)])
+def test_wta_loads_ties_and_special_values(d, off, dtype):
+    w, h = 37, 5
+    rng = np.random.default_rng(7 * d + off)
+    tdt, flag = (torch.float32, Z.ZNCC_F32) if dtype == "f32" else (torch.float16, Z.ZNCC_F16)
+    v = rng.integers(-3, 4, (h, w, d)).astype(np.float32)            # many ties
+    v[0, 0] = -np.inf                                                # nothing beats the start: 0
+    v[0, 1] = np.nan
+    v[1, :, d // 2:] = -np.inf
+    v[2, :, ::2] = np.nan
+    v[3] = np.where(v[3] == 0, -0.0, v[3])
+    buf = torch.zeros(off + h * w * d, dtype=tdt, device="cuda")
+    cost = buf[off:].view(h, w, d)
+    cost.copy_(torch.from_numpy(v))
+    disp = torch.empty((h, w), dtype=torch.int16, device="cuda")
+    with Z.ZnccContext(w, h, d, 3) as ctx:
+        ctx.wta_disparity(cost, disp, flag)
+        torch.cuda.synchronize()
+    n = np.where(np.isnan(v), -np.inf, v)
+    ref = np.where(n.max(-1) == -np.inf, 0, n.argmax(-1))            # argmax: the smallest d of a tie
+    assert np.array_equal(disp.cpu().numpy(), ref)
