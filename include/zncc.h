@@ -344,19 +344,18 @@ const char* zncc_status_string(zncc_status status);
  *                        TMA unit) where both images and the pitch are 16-byte aligned and W is
  *                        a multiple of 16, plain loads elsewhere
  *   ZNCC_TUNE_V_LPC      vertical DT pairs that store the volume: at most this many adjacent
- *                        columns per block (1, 2 or 4; 0 = automatic, which prefers two
- *                        resident blocks per SM). Adjacent columns of a row share DRAM pages,
+ *                        columns per block (1, 2 or 4; 0 = automatic). Adjacent columns of a row share DRAM pages,
  *                        so wider groups make longer runs per page at the cost of residency;
  *                        the last vertical pair with WTA keeps the automatic shape
- *   ZNCC_TUNE_LINE_LOADS DT pairs: 1 = stream the next slices into shared memory with 16-byte
- *                        cp.async per thread and position; 0 (automatic) = in the horizontal
- *                        pairs one TMA tensor copy per 16-position chunk and slice, completing
- *                        on per-warp mbarriers, where the volume and its pixel stride are
- *                        16-byte aligned, F32 or F16 reads span at most four chunks per
- *                        shared-memory wavefront, a line fits one CTA and shared memory allows;
- *                        cp.async elsewhere and in the vertical pairs; 2 = TMA in the vertical
- *                        pairs too (a column box fetches one pixel row at a time: faster for
- *                        some shapes, far slower for others)
+ *   ZNCC_TUNE_LINE_LOADS DT pairs: 0 (automatic) = the fused runs with F32 and F16 storage keep
+ *                        their volume in slabs of 64 bytes per pixel and bring each step's
+ *                        16-position chunks into shared memory by TMA tensor copies; elsewhere
+ *                        (I8 storage, dt_aggregate) one TMA copy per chunk and slice in the
+ *                        horizontal pairs where the volume and its pixel stride are 16-byte
+ *                        aligned, F32 or F16 reads span at most four chunks per shared-memory
+ *                        wavefront, a line fits one CTA and shared memory allows, 16-byte cp.async
+ *                        otherwise; 1 = the volume as [H][W][D], cp.async only; 2 = the volume as
+ *                        [H][W][D], TMA in both directions. The maps do not depend on it
  *   ZNCC_TUNE_WAIT_DRILL (tests) 1 = every DT pair launch has one thread per block wait, with a
  *                        64-poll limit, for an mbarrier phase that nothing completes; the wait
  *                        runs out and records fault bit 2 (see zncc_device_faults) while the

@@ -38,6 +38,8 @@ def _units():
     """(source, object, extra flags) for every translation unit."""
     units = [(os.path.join(CSRC, "api.cu"), "api.o", []),
              (os.path.join(CSRC, "kernels.cu"), "kernels.o", []),
+             (os.path.join(CSRC, "dt_lines.cu"), "dt_lines_f32.o", []),
+             (os.path.join(CSRC, "dt_lines.cu"), "dt_lines_f16.o", ["-DDT_LINES_F16"]),
              (os.path.join(CSRC, "static_scratch.cu"), "static_scratch.o", []),
              (os.path.join(CSRC, "plane.cu"), "plane.o", []),
              (os.path.join(CSRC, "serve.cpp"), "serve.o", [])]

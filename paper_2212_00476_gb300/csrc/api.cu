@@ -118,7 +118,7 @@ struct zncc_ctx {
     struct TmapEntry {
         const void* base;
         long long dstride;
-        int elem, horiz, ds, np;
+        int elem, horiz, ds, np, lines;             // lines: 0 for k_line_pair's 3-D maps
         CUtensorMap map;
     };
     std::vector<TmapEntry> tmaps;
@@ -294,6 +294,9 @@ zncc_status alloc_dev(zncc_ctx* c, void** p, size_t bytes, const char* what) {
     return ZNCC_OK;
 }
 
+// The sd_shift of a volume in one slab.
+constexpr int kOneSlab = 30;
+
 // One pair of a (possibly batched) call: its context and this call's buffers. lc, the
 // launching context, is the first pair's: its stream carries every launch, and errors and
 // per-kernel timings are recorded on it.
@@ -303,8 +306,9 @@ struct PairIO {
     const uint8_t* right;
     int pitch;
     uint16_t* disp;
-    void* vol;              // the pair's cost volume [H][W][dstride]
-    long long dstride;
+    void* vol;              // the pair's cost volume: [H][W][dstride], or slabs of dstride = 2^sd_shift
+    long long dstride;      // disparities (sd_shift < kOneSlab), [slab][H][W][dstride]
+    int sd_shift = kOneSlab;
     const float2* mulmap1 = nullptr;     // (FastDT) the multipliers of the cost kernel's pass pair
 };
 
@@ -377,7 +381,8 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
             a.d_hi = c->D;
             a.vol = io[i].vol;
             a.dstride = io[i].dstride;
-            a.d_out0 = 0;
+            a.sd_shift = io[i].sd_shift;
+            a.slab_stride = (long long)c->W * c->H * io[i].dstride;
             a.vec = io[i].vol && (io[i].dstride % 4 == 0) &&
                     ((uintptr_t)io[i].vol % (dtype == 0 ? 16 : (dtype == 1 ? 8 : 4)) == 0) ? 1 : 0;
             a.mulmap = io[i].mulmap1;
@@ -441,6 +446,8 @@ struct LinePass {
     unsigned long long* keys = nullptr;   // (Wta)
     float s2 = 1.0f;
     int force_tq = 0;
+    int sd_shift = kOneSlab;          // slabs of dstride = 2^sd_shift disparities (k_dt_lines only)
+    int v_lpc = 0;                    // most lines per block of a vertical store pass (0: automatic)
 };
 
 // The block shape of a pair's pass: among lane counts per chunk (8, 4, 2, or the forced
@@ -632,7 +639,7 @@ bool line_tma(zncc_ctx* c, const LineArgs& a, const LinePass& p, CUtensorMap& m)
     const cuuint32_t ds = (cuuint32_t)(kG * a.tq), np = (cuuint32_t)(kL + g - 1);
     for (const zncc_ctx::TmapEntry& t : c->tmaps)
         if (t.base == in && t.dstride == p.dstride && t.elem == (int)elem && t.horiz == (int)p.horiz &&
-            t.ds == (int)ds && t.np == (int)np) {
+            t.ds == (int)ds && t.np == (int)np && t.lines == 0) {
             m = t.map;
             return true;
         }
@@ -647,7 +654,7 @@ bool line_tma(zncc_ctx* c, const LineArgs& a, const LinePass& p, CUtensorMap& m)
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
     if (c->tmaps.size() >= 32) c->tmaps.clear();   // (callers' own volumes, e.g. dt_aggregate)
-    c->tmaps.push_back(zncc_ctx::TmapEntry{in, p.dstride, (int)elem, (int)p.horiz, (int)ds, (int)np, m});
+    c->tmaps.push_back(zncc_ctx::TmapEntry{in, p.dstride, (int)elem, (int)p.horiz, (int)ds, (int)np, 0, m});
     return true;
 }
 
@@ -674,12 +681,177 @@ void add_line_pair(LineBatch& b, const LineArgs& ai, int mode, int dtype, int& t
     rest = std::max(rest, line_pair_smem_bytes(mode, dtype, a, line_coef_async(a)) - st);
 }
 
+// The block shape of a pass for k_dt_lines, whose carries associate in groups of `scan` chunks;
+// false where no shape fits.
+//  - lanes per chunk: the most whose disparities a pixel of a slab holds and whose scan group
+//    lies in a warp: 8 lanes read whole 128-byte lines of shared memory (4 lanes take two
+//    wavefronts) and step over twice the disparities per barrier (F16 rows of 1242 pixels:
+//    90 us a pass with 4 lanes, 66 with 8).
+//  - lines per block: columns in fours for 64-byte pixels, so that a row of the box is 256
+//    bytes of DRAM (1280x384x128 F32, columns per block: 4 88.9 us, 2 89.7, 1 104), rows one
+//    by one (a row's slab is contiguous anyway). Blocks of more than 512 threads get 96
+//    registers a thread instead of 128; a store pass in F32 loses more by that than two columns
+//    gain (columns of 1080: one column per block 752 us, two in 576 threads 797), the WTA pass
+//    and half storage gain (WTA there: 653 and 504 us).
+//  - coefficient buffers per line: two where they fit, so that a group's coefficients arrive
+//    during the one before.
+bool dt_lines_shape(const zncc_ctx* c, const LinePass& p, int scan, DtShape& best) {
+    const int n = p.horiz ? c->W : c->H, elem = p.dtype == 0 ? 4 : 2;
+    const int most = p.mode == kLineWta || p.dtype == 1 ? kDtThreads : 512;
+    for (int lanes = 8; lanes >= 2; lanes /= 2) {
+        const int nch = padded_chunks(n, lanes), per_line = nch * lanes;
+        if (scan * lanes > 32 || per_line > most || kG * lanes > (1 << p.sd_shift)) continue;
+        int lines = p.horiz ? 1 : 256 / (kG * lanes * elem);
+        if (p.v_lpc > 0 && !p.horiz && p.mode == kLineStore) lines = std::min(lines, p.v_lpc);
+        for (; lines >= 1; --lines) {
+            if (lines * per_line > most) continue;
+            for (int nco = 2; nco >= 1; --nco) {
+                DtShape s{lanes, scan, lines, nch, nco, p.horiz ? 1 : 0};
+                if (dt_lines_layout(p.dtype, p.mulmap != nullptr, s) > (size_t)c->smem_max) continue;
+                best = s;
+                return true;
+            }
+        }
+    }
+    return false;
+}
+
+// The tensor map of a pass's volume for k_dt_lines: {entries per pixel and slab, W, H, slabs}.
+bool dt_lines_tmap(zncc_ctx* c, const LinePass& p, const DtShape& s, CUtensorMap& m) {
+    const long long elem = p.dtype == 0 ? 4 : 2;
+    const int ds = kG * s.lanes;
+    for (const zncc_ctx::TmapEntry& t : c->tmaps)
+        if (t.base == p.vol && t.dstride == p.dstride && t.elem == (int)elem && t.horiz == (int)p.horiz &&
+            t.ds == ds && t.np == p.sd_shift && t.lines == s.lines) {
+            m = t.map;
+            return true;
+        }
+    const TmapEncodeFn enc = tmap_encoder();
+    if (!enc) return false;
+    const cuuint64_t slabs = p.sd_shift == kOneSlab ? 1 : (cuuint64_t)((p.dcount + p.dstride - 1) / p.dstride);
+    const cuuint64_t dims[4] = {(cuuint64_t)p.dstride, (cuuint64_t)c->W, (cuuint64_t)c->H, slabs};
+    const cuuint64_t row = (cuuint64_t)(p.dstride * elem);
+    const cuuint64_t strides[3] = {row, row * c->W, row * c->W * c->H};
+    const cuuint32_t box[4] = {(cuuint32_t)ds, (cuuint32_t)(p.horiz ? kL : s.lines),
+                               (cuuint32_t)(p.horiz ? s.lines : kL), 1u};
+    const cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
+    if (enc(&m, p.dtype == 0 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, p.vol, dims,
+            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    if (c->tmaps.size() >= 32) c->tmaps.clear();
+    c->tmaps.push_back(zncc_ctx::TmapEntry{p.vol, p.dstride, (int)elem, (int)p.horiz, ds, p.sd_shift, s.lines, m});
+    return true;
+}
+
+// k_dt_lines launches over the passes of several pairs: those of the same block shape share one.
+zncc_status run_dt_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* passes, const DtShape* shapes,
+                         const CUtensorMap* tmaps, int n, int kind) {
+    const int mode = passes[0].mode, dtype = passes[0].dtype;
+    bool done[kMaxBatch] = {false};
+    for (int first = 0; first < n; ++first) {
+        if (done[first]) continue;
+        const DtShape& s = shapes[first];
+        const bool alone = fills_device(ctxs[first]);
+        DtBatch<kMaxBatch> b;
+        b.npairs = b.total_steps = 0;
+        b.s = s;
+        b.s2 = passes[first].s2;
+        b.fault = lc->fault;
+        b.drill = lc->wait_drill;
+        for (int i = first; i < n; ++i) {
+            const DtShape& t = shapes[i];
+            if (done[i] || t.lanes != s.lanes || t.scan != s.scan || t.lines != s.lines || t.nch != s.nch ||
+                t.nco != s.nco || (i != first && (alone || fills_device(ctxs[i]))))
+                continue;
+            done[i] = true;
+            const zncc_ctx* c = ctxs[i];
+            const LinePass& p = passes[i];
+            const int W = c->W, H = c->H;
+            b.tmap[b.npairs] = tmaps[i];
+            DtArgs& a = b.p[b.npairs++];
+            a.vol = p.vol;
+            a.pos_stride = p.horiz ? p.dstride : (long long)W * p.dstride;
+            a.line_stride = p.horiz ? (long long)W * p.dstride : p.dstride;
+            a.slab_stride = (long long)W * H * p.dstride;
+            a.sd_shift = p.sd_shift;
+            a.n = p.horiz ? W : H;
+            a.nlines = p.horiz ? H : W;
+            a.dcount = p.dcount;
+            a.mulmap = p.mulmap;
+            a.coef = p.horiz ? c->coefH : c->coefV;
+            a.keys = p.keys;
+            a.pix_line = p.horiz ? W : 1;
+            a.pix_pos = p.horiz ? 1 : W;
+            const int ds = kG * s.lanes;
+            a.step0 = b.total_steps;
+            a.nsl = (a.dcount + ds - 1) / ds;
+            a.ngroups = (a.nlines + s.lines - 1) / s.lines;
+            b.total_steps += a.ngroups * a.nsl;
+        }
+        const size_t smem = dt_lines_layout(dtype, passes[first].mulmap != nullptr, b.s);
+        const int threads = s.lines * s.nch * s.lanes;
+        int bps = 0;
+        ZNCC_CUDA(lc, cached_occupancy(lc, 4, (((long long)mode * 4 + dtype) * 16 + s.lanes) * 2 + (b.npairs == 1), (long long)smem * 1024 + threads,
+                                       [&](int* v) {
+                                           return (dtype == 0 ? dt_lines_occupancy_f32 : dt_lines_occupancy_f16)(
+                                               mode, s.lanes, threads, smem, b.npairs == 1, v);
+                                       },
+                                       &bps), "occupancy query");
+        b.grid = std::max(1, std::min(b.total_steps, lc->num_sms * std::max(1, bps)));
+        ZNCC_LAUNCH(lc, kind, (dtype == 0 ? launch_dt_lines_f32 : launch_dt_lines_f16)(b, smem, mode, lc->cur), "DT pass pair");
+    }
+    return ZNCC_OK;
+}
+
+// The chunks per scan group of a pass: those that a warp holds in k_line_pair's block shape for
+// it (p.vol may be NULL: the volume is then taken to be aligned). 0 where it has none.
+int dt_scan_group(zncc_ctx* c, const LinePass& p) {
+    LineArgs a;
+    LinePass q = p;
+    q.dstride = (p.dcount + 3) / 4 * 4;
+    fill_line_args(a, q, c->W, c->H, c->coefH, c->coefV);
+    return plan_line_pass(c, a, q) == ZNCC_OK ? 32 / a.tq : 0;
+}
+
+// Whether the fused path of a pair keeps its volume in slabs and runs every line pass in k_dt_lines.
+// Slabs of 64 bytes per pixel: a row of a slab is contiguous, and an H pass reads and writes
+// whole pixels of it step by step.
+int slab_shift(int dtype) { return dtype == 0 ? 4 : 5; }
+const float2 kSomeMul{};          // stands for a multiplier map where only its presence counts
+
+bool slab_path(zncc_ctx* c, int dtype, bool norm) {
+    if (c->line_loads != 0 || dtype == 2 || !tmap_encoder()) return false;
+    for (int k = 0; k < 3; ++k) {                   // rows, columns, columns with WTA
+        LinePass p;
+        p.dcount = c->D;
+        p.dtype = dtype;
+        p.horiz = k == 0;
+        p.mode = k == 2 ? kLineWta : kLineStore;
+        p.mulmap = norm ? &kSomeMul : nullptr;
+        p.sd_shift = slab_shift(dtype);
+        p.v_lpc = c->v_lpc;
+        DtShape s;
+        const int scan = dt_scan_group(c, p);
+        if (!scan || !dt_lines_shape(c, p, scan, s)) return false;
+    }
+    return true;
+}
+
 // Line-pair launches over the passes of several pairs (the same mode and storage): pairs
 // whose passes have the same block shape share one launch.
 zncc_status run_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* passes, int n, int kind) {
     const int mode = passes[0].mode, dtype = passes[0].dtype;
     LineArgs args[kMaxBatch];
     CUtensorMap tmaps[kMaxBatch];
+    if (passes[0].sd_shift != kOneSlab) {           // (every pair's volume is in slabs)
+        DtShape shapes[kMaxBatch];
+        for (int i = 0; i < n; ++i)
+            if (!dt_lines_shape(ctxs[i], passes[i], dt_scan_group(ctxs[i], passes[i]), shapes[i]) ||
+                !dt_lines_tmap(ctxs[i], passes[i], shapes[i], tmaps[i]))
+                return fail(lc, ZNCC_EUNSUPPORTED, "DT pass: no block shape or tensor map");
+        return run_dt_lines(lc, ctxs, passes, shapes, tmaps, n, kind);
+    }
     for (int i = 0; i < n; ++i) {
         zncc_ctx* c = ctxs[i];
         const LinePass& p = passes[i];
@@ -895,10 +1067,18 @@ zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigm
     }
     const int dt = storage;                         // 0 float, 1 half, 2 FastDT codes
     zncc_ctx* ctxs[kMaxBatch];
+    bool slabs = true;
+    for (int i = 0; i < n; ++i) slabs = slabs && slab_path(io[i].c, dt, dt == 1 && iters > 1);
     for (int i = 0; i < n; ++i) {
         ctxs[i] = io[i].c;
         io[i].dstride = (io[i].c->D + 3) / 4 * 4;     // padded so that every access is vectorised
-        if (ensure_volume(io[i].c, dt, io[i].dstride) != ZNCC_OK) return fail(lc, ZNCC_ENOMEM, io[i].c->err);
+        long long entries = io[i].dstride;
+        if (slabs) {
+            io[i].sd_shift = slab_shift(dt);
+            io[i].dstride = 1 << io[i].sd_shift;
+            entries = (io[i].c->D + io[i].dstride - 1) / io[i].dstride * io[i].dstride;
+        }
+        if (ensure_volume(io[i].c, dt, entries) != ZNCC_OK) return fail(lc, ZNCC_ENOMEM, io[i].c->err);
         io[i].vol = io[i].c->vol;
     }
     const float K = (float)exp(-1.0 / (double)sigma_s);
@@ -1006,6 +1186,8 @@ zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigm
             const size_t npix = (size_t)io[i].c->W * io[i].c->H;
             lp[i].vol = io[i].vol;
             lp[i].dstride = io[i].dstride;
+            lp[i].sd_shift = io[i].sd_shift;
+            lp[i].v_lpc = io[i].c->v_lpc;
             lp[i].dcount = io[i].c->D;
             lp[i].dtype = dt;
             lp[i].s2 = s2;

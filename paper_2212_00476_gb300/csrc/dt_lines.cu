@@ -1,0 +1,451 @@
+// dt_lines.cu -- the DT pass pair along rows or columns (Sec. III-B, Eqs. (3)-(6)) over a volume
+// in disparity slabs, F32 or F16 storage, with the WTA fused into the last pair (Sec. V-C).
+#include <algorithm>
+#include <type_traits>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace zncc {
+
+// ---------------------------------------------------------------------------------------
+// A thread holds 16 consecutive positions (a chunk) x 4 disparities in registers; `lanes`
+// lanes share a chunk, so a step is 4 * lanes disparities of `lines` adjacent lines. The block
+// takes the steps [s0, s1) of all (line group, disparity slice) in order, slices innermost.
+//
+// The result of a pass depends, in its last bits, on how the chunks' affine maps are composed:
+// in scan groups of `scan` consecutive chunks by doubling rounds, then group by group. The scan
+// group is given by the caller and does not depend on the lanes per chunk, so a shape can be
+// chosen for speed alone.
+//
+// Bound by HBM for F32 store passes: a pass moves the volume once in and once out, and an
+// in-place pass of a plain kernel over the same bytes takes 78-82 us at 1280x384x128. Measured
+// there (k_line_pair -> this kernel, us): columns 94 -> 89, rows 95 -> 85, last columns with WTA
+// 75 -> 63; F16 at 1242x375x128: columns 77 -> 60, rows 110 -> 64, WTA 84 -> 53; F32 at
+// 1920x1080x256: columns 1188 -> 731, rows 888 -> 710, WTA 790 -> 506.
+//
+// Staging: one lane per chunk copies the box of the next step's chunk (all lines of the group)
+// into shared memory by TMA as soon as the lines' warps have read the last one into registers,
+// so that the copy is in flight during the whole step. A warp waits for its own chunks only
+// (an mbarrier per warp of a line), and the two barriers of the pass pair are per line: the
+// lines of a block share nothing but their boxes.
+template <bool SCALE, int lanes, typename Hook>
+__device__ __forceinline__ void dt_lines_pair(float (&v)[kL][4], const float4* __restrict__ co, int scan_shift, int lane,
+                                              int k, int nvg, float* sa, float4* sb, float s2,
+                                              const float2* __restrict__ mul, int bar, int bar_threads,
+                                              Hook after_read) {
+    const int scan = 1 << scan_shift, c = k & (scan - 1), vg = k >> scan_shift;     // place in the scan group, scan group
+    // ---- phase 1: forward sweep of the chunk with zero carry-in, scan of the group's maps ----
+    {
+        float u[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < kL; ++i) {
+            fma4<true>(co[i].x, u, v[i], u);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[i][j] = u[j];
+        }
+    }
+    after_read();
+    float A = co[kL - 1].y, B[4], Ae, Be[4], F[4], G[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        B[j] = v[kL - 1][j];
+        F[j] = G[j] = 0.0f;
+    }
+#pragma unroll
+    for (int r = 0; (lanes << r) < 32; ++r) {
+        const int off = lanes << r;
+        if ((1 << r) >= scan) break;
+        const float A2 = __shfl_up_sync(kFull, A, off);
+        float B2[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) B2[j] = __shfl_up_sync(kFull, B[j], off);
+        if (c >= (1 << r)) {
+            fma4<true>(A, B2, B, B);
+            A *= A2;
+        }
+    }
+    Ae = __shfl_up_sync(kFull, A, lanes);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) Be[j] = __shfl_up_sync(kFull, B[j], lanes);
+    if (c == 0) {
+        Ae = 1.0f;
+        Be[0] = Be[1] = Be[2] = Be[3] = 0.0f;
+    }
+    if (c == scan - 1) {
+        sa[vg * lanes] = A;
+        sb[vg * lanes] = make_float4(B[0], B[1], B[2], B[3]);
+    }
+    named_barrier(bar, bar_threads);
+
+    // ---- phase 2: carry from the groups before, corrected forward values, backward sweep ----
+#pragma unroll 1
+    for (int g = 0; g < vg; ++g) {
+        const float4 b2 = sb[g * lanes];
+        const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
+        fma4<true>(sa[g * lanes], F, b4, F);
+    }
+    fma4<true>(Ae, F, Be, F);
+    float h[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = kL - 1; i >= 0; --i) {
+        const float4 w = co[i];
+        float ft[4];
+        fma4<true>(w.y, F, v[i], ft);
+        fma4<true>(w.z, h, ft, h);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[i][j] = h[j];
+    }
+    A = co[0].w;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) B[j] = h[j];
+#pragma unroll
+    for (int r = 0; (lanes << r) < 32; ++r) {
+        const int off = lanes << r;
+        if ((1 << r) >= scan) break;
+        const float A2 = __shfl_down_sync(kFull, A, off);
+        float B2[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) B2[j] = __shfl_down_sync(kFull, B[j], off);
+        if (c + (1 << r) < scan) {
+            fma4<true>(A, B2, B, B);
+            A *= A2;
+        }
+    }
+    Ae = __shfl_down_sync(kFull, A, lanes);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) Be[j] = __shfl_down_sync(kFull, B[j], lanes);
+    if (c == scan - 1) {
+        Ae = 1.0f;
+        Be[0] = Be[1] = Be[2] = Be[3] = 0.0f;
+    }
+    float* sa2 = sa + nvg * lanes;
+    float4* sb2 = sb + nvg * lanes;
+    if (c == 0) {
+        sa2[vg * lanes] = A;
+        sb2[vg * lanes] = make_float4(B[0], B[1], B[2], B[3]);
+    }
+    named_barrier(bar, bar_threads);
+
+    // ---- phase 3: carry from the groups after, backward correction, scale ----
+#pragma unroll 1
+    for (int g = nvg - 1; g > vg; --g) {
+        const float4 b2 = sb2[g * lanes];
+        const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
+        fma4<true>(sa2[g * lanes], G, b4, G);
+    }
+    fma4<true>(Ae, G, Be, G);
+    if (SCALE && (mul || s2 != 1.0f)) {
+#pragma unroll
+        for (int i = 0; i < kL; ++i) {
+            fma4<true>(co[i].w, G, v[i], v[i]);
+            mul4<true>(mul ? mul[i].y : s2, v[i]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kL; ++i) fma4<true>(co[i].w, G, v[i], v[i]);
+    }
+}
+
+// The WTA of a step (Eq. (WTA1)): each thread takes the best of its four disparities at each
+// of its 16 positions, the chunk's lanes merge theirs by halving rounds (WtaRegs::merge), and
+// a lane keeps the running best of the 16 / lanes positions that it ends up with: a few
+// registers where a running best of all 16 positions took 24 (which spilled).
+template <int lanes>
+struct StepWta {
+    static constexpr int kHeld = kL / lanes;
+    float rv[kHeld];
+    int rd[kHeld];
+    __device__ __forceinline__ void reset() {
+#pragma unroll
+        for (int k = 0; k < kHeld; ++k) {
+            rv[k] = -INFINITY;
+            rd[k] = 0x7FFFFFFF;
+        }
+    }
+    // slices arrive in increasing d, so that a later equal value does not replace an earlier one
+    __device__ __forceinline__ void fold(float (&v)[kL][4], int nvalid, int d_first, int dq) {
+        if (nvalid < 4) {
+#pragma unroll
+            for (int i = 0; i < kL; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (j >= nvalid) v[i][j] = -INFINITY;
+        }
+        float bv[kL];
+        int bd[kL];
+#pragma unroll
+        for (int i = 0; i < kL; ++i) {
+            const float m01 = fmaxf(v[i][0], v[i][1]), m23 = fmaxf(v[i][2], v[i][3]);
+            const bool lo = m01 >= m23;
+            bv[i] = lo ? m01 : m23;
+            bd[i] = d_first + (lo ? (v[i][0] >= v[i][1] ? 0 : 1) : (v[i][2] >= v[i][3] ? 2 : 3));
+        }
+        wta_halve<16>(bv, bd, (dq & 1) != 0, 1);
+        if constexpr (lanes > 2) wta_halve<8>(bv, bd, (dq & 2) != 0, 2);
+        if constexpr (lanes > 4) wta_halve<4>(bv, bd, (dq & 4) != 0, 4);
+#pragma unroll
+        for (int k = 0; k < kHeld; ++k)
+            if (bv[k] > rv[k]) {
+                rv[k] = bv[k];
+                rd[k] = bd[k];
+            }
+    }
+    // the first of the positions that lane dq holds
+    __device__ __forceinline__ static int first(int dq) {
+        return ((dq & 1) ? 8 : 0) + ((dq & 2) ? 4 : 0) + ((dq & 4) ? 2 : 0);
+    }
+};
+
+template <typename T, int MODE, int lanes, int NP, int MAXT>
+__global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBatch<NP> b) {
+    constexpr bool SINGLE = NP == 1;
+    constexpr int ds = kG * lanes, cpw = 32 / lanes;     // disparities per step, chunks per warp
+    extern __shared__ __align__(128) unsigned char dt_smem[];
+    __shared__ unsigned long long full[kDtThreads / 32], empty[kDtThreads / 32], drill_bar;
+    if (threadIdx.x < b.s.nwl) {            // per warp of a line: its chunks' boxes, their readers
+        mbar_init(&full[threadIdx.x], (unsigned)cpw);
+        mbar_init(&empty[threadIdx.x], (unsigned)b.s.lines);
+    }
+    // (tests) the wait drill, as in k_line_pair
+    if (b.drill && threadIdx.x == 0) mbar_init(&drill_bar, 1);
+    __syncthreads();
+    if (b.drill && threadIdx.x == 0 && !mbar_wait(&drill_bar, 0, kDrillWaitPolls)) atomicOr(b.fault, kFaultTmaWait);
+    griddep_wait();
+
+    auto P = [&](int pi) -> const DtArgs& { return b.p[SINGLE ? 0 : pi]; };
+    // A step: the pair, the line group and the slice. Of one pair's groups the blocks take whole
+    // ones in turn (block i the groups i, i + grid, ...), so that the blocks are at adjacent
+    // lines at any time and their short runs of a pixel row fall together in DRAM; the groups
+    // that do not fill a round, and the groups of several pairs, go by equal ranges of steps.
+    struct Cursor {
+        int pi, g, sl;
+    };
+    const int full_rounds = SINGLE ? b.p[0].ngroups / b.grid * b.grid : 0;        // groups taken in turn
+    Cursor rest;                            // the block's first step among the others
+    int left;                               // steps from the cursor to the end of the block's
+    {
+        const int first = full_rounds * (SINGLE ? b.p[0].nsl : 0), others = b.total_steps - first;
+        const int s0 = first + (int)((long long)blockIdx.x * others / b.grid);
+        left = first + (int)((long long)(blockIdx.x + 1) * others / b.grid) - s0;
+        rest.pi = 0;
+        if (!SINGLE)
+            while (rest.pi + 1 < b.npairs && s0 >= b.p[rest.pi + 1].step0) ++rest.pi;
+        rest.g = (s0 - P(rest.pi).step0) / P(rest.pi).nsl;
+        rest.sl = s0 - P(rest.pi).step0 - rest.g * P(rest.pi).nsl;
+        left += first / b.grid;
+    }
+    auto next_group = [&](Cursor& q) {
+        q.sl = 0;
+        if (SINGLE && q.g < full_rounds) {
+            q.g += b.grid;
+            if (q.g >= full_rounds) q = rest;
+        } else if (++q.g == P(q.pi).ngroups && !SINGLE && q.pi + 1 < b.npairs) {
+            q.g = 0;
+            ++q.pi;
+        }
+    };
+    auto advance = [&](Cursor& q) {
+        if (++q.sl == P(q.pi).nsl) next_group(q);
+    };
+    Cursor o = rest;
+    if (SINGLE && full_rounds > 0) o = Cursor{0, (int)blockIdx.x, 0};
+
+    // this thread's place: line li of the group, warp w of the line, chunk k, lane dq of the chunk
+    const int li = threadIdx.x / b.s.per_line;
+    const int w = (threadIdx.x - li * b.s.per_line) >> 5;
+    const int lane = threadIdx.x & 31;
+    const int dq = lane & (lanes - 1), k = w * cpw + lane / lanes;
+    // shared memory: [staging][coefficients: nco per line][multipliers: nco][scan buffers]
+    unsigned char* const base = dt_smem + (-smem_addr(dt_smem) & 127u);      // (a tensor copy's alignment)
+    const T* const mine = reinterpret_cast<T*>(base) + k * b.s.slot + li * b.s.line_off + dq * kG;
+    float4* const co_mine = reinterpret_cast<float4*>(base + b.s.co_off) + li * b.s.nco * b.s.arr;     // this line's
+    float2* const mul_mine = reinterpret_cast<float2*>(base + b.s.mul_off) + li * b.s.nco * b.s.arr;
+    float4* const sb = reinterpret_cast<float4*>(base + b.s.scan_off) + li * 2 * b.s.nvg * lanes + dq;
+    float* const sa = reinterpret_cast<float*>(base + b.s.scan_off + b.s.lines * 2 * b.s.nvg * lanes * 16) +
+                      li * 2 * b.s.nvg * lanes + dq;
+
+    auto prefetch_coef = [&](const Cursor& q, int cbuf) {
+        const DtArgs& a = P(q.pi);
+        const int ln = q.g * b.s.lines + li;
+        for (int t = w * 32 + lane; t < b.s.nch * kL; t += b.s.per_line) {
+            const bool in = ln < a.nlines && t < a.n;
+            const size_t at = (size_t)ln * a.n + t;
+            cp_async<16>(co_mine + cbuf * b.s.arr + cpos(t), in ? a.coef + at : a.coef, in);
+            if (b.s.mul) cp_async<8>(mul_mine + cbuf * b.s.arr + cpos(t), in ? a.mulmap + at : a.mulmap, in);
+        }
+        cp_async_commit();
+    };
+    // the box of this chunk at the step of cursor q (lines past the pass, positions past the
+    // line and disparities past the volume read as zero)
+    auto load_box = [&](const Cursor& q) {
+        const int d0 = q.sl * ds, sd_shift = P(q.pi).sd_shift;
+        const int slab = d0 >> sd_shift, dd = d0 & ((1 << sd_shift) - 1);
+        unsigned long long* bar = &full[w];
+        T* dst = reinterpret_cast<T*>(base) + k * b.s.slot;
+        fence_proxy_async_smem();
+        mbar_expect_tx(bar, (unsigned)(b.s.slot * sizeof(T)));
+        const CUtensorMap* m = &b.tmap[SINGLE ? 0 : q.pi];
+        const int at = k * kL, line0 = q.g * b.s.lines;
+        tma_load_4d(dst, m, dd, b.s.horiz ? at : line0, b.s.horiz ? line0 : at, slab, bar);
+    };
+    if (li == 0 && dq == 0 && left > 0) load_box(o);
+    if (b.s.nco == 2) prefetch_coef(o, 0);
+
+    StepWta<lanes> wr;
+    int cbuf = b.s.nco - 1;
+    bool fresh = true;
+    for (unsigned par = 0; left > 0; par ^= 1u, --left) {
+        const DtArgs& a = P(o.pi);
+        if (left == 1) griddep_launch_dependents();
+        if (fresh) {                            // a new line group: its coefficients
+            if (b.s.nco == 1) {                 // one buffer: filled once its readers are done
+                named_barrier(1 + li, b.s.per_line);
+                prefetch_coef(o, 0);
+            }
+            cp_async_wait<0>();
+            named_barrier(1 + li, b.s.per_line);
+            if (b.s.nco == 2) {                 // two: the next group's arrive during this one
+                cbuf ^= 1;
+                if (left > a.nsl - o.sl) {
+                    Cursor nx = o;
+                    next_group(nx);
+                    prefetch_coef(nx, cbuf ^ 1);
+                }
+            }
+            if constexpr (MODE == kLineWta) wr.reset();
+        }
+        const float4* co = co_mine + cbuf * b.s.arr + k * kCS;
+        const float2* mul = b.s.mul ? mul_mine + cbuf * b.s.arr + k * kCS : nullptr;
+        if (!mbar_wait(&full[w], par, kBulkWaitPolls)) {       // (a timeout is recorded, then waited
+            atomicOr(b.fault, kFaultTmaWait);                   // for once more)
+            mbar_wait(&full[w], par, kBulkWaitPolls);
+        }
+        float v[kL][4];
+#pragma unroll
+        for (int i = 0; i < kL; ++i) lds4(mine + i * b.s.ps, v[i]);
+        if (b.s.mul) {
+#pragma unroll
+            for (int i = 0; i < kL; ++i) mul4<true>(mul[i].x, v[i]);
+        }
+        dt_lines_pair<MODE != kLineWta, lanes>(v, co, b.s.scan_shift, lane, k, b.s.nvg, sa, sb, b.s2, mul, 1 + li, b.s.per_line,
+            [&]() {
+                // the box has been read: the lines' warps say so, and its loader refills it
+                __syncwarp();
+                if (b.s.lines > 1 && lane == 0) mbar_arrive(&empty[w]);
+                if (li == 0 && dq == 0 && left > 1) {
+                    if (b.s.lines > 1 && !mbar_wait(&empty[w], par, kBulkWaitPolls)) {
+                        atomicOr(b.fault, kFaultTmaWait);
+                        mbar_wait(&empty[w], par, kBulkWaitPolls);
+                    }
+                    Cursor q = o;
+                    advance(q);
+                    load_box(q);
+                }
+            });
+        const int dl = o.sl * ds + dq * kG;
+        const int nvalid = max(0, min(4, a.dcount - dl));
+        const int line = o.g * b.s.lines + li;
+        if constexpr (MODE == kLineWta) {
+            wr.fold(v, nvalid, dl, dq);
+            if (o.sl == a.nsl - 1 || left == 1) {
+#pragma unroll
+                for (int i = 0; i < wr.kHeld; ++i) {
+                    const int pos = k * kL + wr.first(dq) + i;
+                    if (line < a.nlines && pos < a.n)
+                        atomicMax(a.keys + (size_t)line * a.pix_line + (size_t)pos * a.pix_pos, wta_key(wr.rv[i], wr.rd[i]));
+                }
+            }
+        } else if (line < a.nlines && nvalid > 0) {
+            const int slab = dl >> a.sd_shift, dd = dl & ((1 << a.sd_shift) - 1), npos = a.n - k * kL;
+            T* q = reinterpret_cast<T*>(a.vol) + slab * a.slab_stride + line * a.line_stride + (k * kL) * a.pos_stride + dd;
+            const long long es = a.pos_stride;
+            if (npos >= kL) {
+#pragma unroll
+                for (int i = 0; i < kL; ++i) st4(q + i * es, 4, true, v[i]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < kL; ++i)
+                    if (i < npos) st4(q + i * es, 4, true, v[i]);
+            }
+        }
+        fresh = o.sl + 1 == a.nsl;
+        advance(o);
+    }
+    cp_async_wait<0>();
+}
+
+#if !defined(DT_LINES_F16)
+size_t dt_lines_layout(int dtype, bool mul, DtShape& s) {
+    const int elem = dtype == 0 ? 4 : 2, ds = kG * s.lanes;
+    s.mul = mul;
+    s.per_line = s.nch * s.lanes;
+    s.nwl = s.per_line / 32;
+    s.nvg = s.nch / s.scan;
+    s.scan_shift = 0;
+    while ((1 << s.scan_shift) < s.scan) ++s.scan_shift;
+    s.slot = s.lines * kL * ds;
+    s.ps = s.horiz ? ds : s.lines * ds;
+    s.line_off = s.horiz ? kL * ds : ds;
+    s.arr = s.nch * kCS;
+    s.co_off = s.nch * s.slot * elem;
+    s.mul_off = s.co_off + s.lines * s.nco * s.arr * 16;
+    s.scan_off = s.mul_off + (mul ? s.lines * s.nco * s.arr * 8 : 0);
+    return 128 + (size_t)s.scan_off + (size_t)s.lines * 2 * s.nvg * s.lanes * 20;
+}
+#define DT_NAME(f) f##_f32
+using DtElem = float;
+#else
+#define DT_NAME(f) f##_f16
+using DtElem = __half;
+#endif
+
+template <int NP, int MAXT>
+static void (*dt_lines_fn_t(int mode, int lanes))(DtBatch<NP>) {
+    if (mode == kLineStore)
+        return lanes == 8   ? k_dt_lines<DtElem, kLineStore, 8, NP, MAXT>
+               : lanes == 4 ? k_dt_lines<DtElem, kLineStore, 4, NP, MAXT>
+                            : k_dt_lines<DtElem, kLineStore, 2, NP, MAXT>;
+    return lanes == 8   ? k_dt_lines<DtElem, kLineWta, 8, NP, MAXT>
+           : lanes == 4 ? k_dt_lines<DtElem, kLineWta, 4, NP, MAXT>
+                        : k_dt_lines<DtElem, kLineWta, 2, NP, MAXT>;
+}
+template <int NP>
+static void (*dt_lines_fn(int mode, int lanes, int threads))(DtBatch<NP>) {
+    return threads <= 512 ? dt_lines_fn_t<NP, 512>(mode, lanes) : dt_lines_fn_t<NP, kDtThreads>(mode, lanes);
+}
+
+cudaError_t DT_NAME(dt_lines_occupancy)(int mode, int lanes, int threads, size_t smem, bool single, int* blocks_per_sm) {
+    const void* fn = single ? (const void*)dt_lines_fn<1>(mode, lanes, threads)
+                            : (const void*)dt_lines_fn<kMaxBatch>(mode, lanes, threads);
+    cudaError_t e = set_max_smem(fn, smem);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
+}
+
+cudaError_t DT_NAME(launch_dt_lines)(const DtBatch<kMaxBatch>& b, size_t smem, int mode, cudaStream_t st) {
+    const int threads = b.s.lines * b.s.nch * b.s.lanes;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    launch_config(cfg, attr, dim3(b.grid), dim3(threads), smem, st, 1);
+    if (b.npairs == 1) {                    // one pair: a small parameter block, read at constant offsets
+        DtBatch<1> o;
+        o.npairs = 1;
+        o.total_steps = b.total_steps;
+        o.grid = b.grid;
+        o.drill = b.drill;
+        o.s2 = b.s2;
+        o.fault = b.fault;
+        o.s = b.s;
+        o.p[0] = b.p[0];
+        o.tmap[0] = b.tmap[0];
+        void (*fn)(DtBatch<1>) = dt_lines_fn<1>(mode, b.s.lanes, threads);
+        cudaError_t e = set_max_smem((const void*)fn, smem);
+        return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, fn, o);
+    }
+    void (*fn)(DtBatch<kMaxBatch>) = dt_lines_fn<kMaxBatch>(mode, b.s.lanes, threads);
+    cudaError_t e = set_max_smem((const void*)fn, smem);
+    return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, fn, b);
+}
+
+}  // namespace zncc

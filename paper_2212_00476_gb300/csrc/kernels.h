@@ -29,7 +29,8 @@ struct RowArgs {
     int spb;                  // disparity slices (4 * tq each) per visit of a row
     void* vol;                // output [H][W][dstride] of float or half (Raw / HPair)
     long long dstride;        // entries per pixel in the output
-    int d_out0;               // disparity stored at entry 0 of a pixel
+    int sd_shift;             // disparity d is entry d mod 2^sd_shift of slab d >> sd_shift ...
+    long long slab_stride;    // ... and a slab is this many entries
     int vec;                  // 16-byte (float) / 8-byte (half) accesses allowed
     float K, inv_sr255;       // DT weights (HPair): exp(-1/sigma_s), 1/(255 sigma_r); guide = left
     float4* coefH_out;        // (HPair) if set, the row coefficients go here too ([H][W], as k_dt_coef)
@@ -109,6 +110,52 @@ struct LineBatch {
     // {4 tq, 16, 1} (rows) or {4 tq, 1, 16} (columns): one chunk's positions of one slice
     CUtensorMap tmap[kMaxBatch];
 };
+
+// The DT pass pair over a volume stored in slabs of sd = 2^sd_shift disparities, [slab][H][W][sd]
+// (one slab of all disparities: a caller's [H][W][D] volume): dt_lines.cu.
+struct DtArgs {
+    void* vol;
+    long long pos_stride;     // entries between consecutive positions of a line
+    long long line_stride;    // entries between consecutive lines
+    long long slab_stride;    // entries between slabs
+    int sd_shift;             // disparity d is entry d mod 2^sd_shift of slab d >> sd_shift
+    int n, nlines, dcount;    // line length, lines, valid disparities
+    const float2* mulmap;     // as LineArgs
+    const float4* coef;
+    unsigned long long* keys; // as LineArgs (Wta)
+    long long pix_line, pix_pos;
+    int step0;                // this pair's first step (line group, disparity slice) in the launch
+    int nsl, ngroups;         // its slices per group and its line groups
+};
+// The block shape of a launch, common to its pairs.
+struct DtShape {
+    int lanes;                // lanes per chunk (4 disparities each): a slice is 4 * lanes disparities
+    int scan;                 // chunks per scan group: the carries' association (a power of two)
+    int lines;                // adjacent lines per block
+    int nch;                  // chunks per line, padded to whole warps
+    int nco;                  // coefficient buffers per line (1 or 2)
+    int horiz;
+    // filled by dt_lines_layout: multipliers in use, threads and warps per line, scan groups per
+    // line, entries of a chunk's box, between its positions and between its lines, of a line's
+    // coefficient array, and byte offsets in shared memory
+    int scan_shift, mul, per_line, nwl, nvg, slot, ps, line_off, arr, co_off, mul_off, scan_off;
+};
+template <int NP>
+struct DtBatch {
+    int npairs, total_steps, grid, drill;
+    float s2;
+    unsigned* fault;
+    DtShape s;
+    DtArgs p[NP];
+    CUtensorMap tmap[NP];     // {sd, W, H, slabs}, box {4 lanes, lines, 16, 1} (columns) or {4 lanes, 16, lines, 1}
+};
+// Completes a shape; returns the dynamic shared memory of its blocks.
+size_t dt_lines_layout(int dtype, bool mul, DtShape& s);
+constexpr int kDtThreads = 640;               // the most threads of a block
+cudaError_t dt_lines_occupancy_f32(int mode, int lanes, int threads, size_t smem, bool single, int* blocks_per_sm);
+cudaError_t dt_lines_occupancy_f16(int mode, int lanes, int threads, size_t smem, bool single, int* blocks_per_sm);
+cudaError_t launch_dt_lines_f32(const DtBatch<kMaxBatch>& b, size_t smem, int mode, cudaStream_t st);
+cudaError_t launch_dt_lines_f16(const DtBatch<kMaxBatch>& b, size_t smem, int mode, cudaStream_t st);
 
 // Launch configuration with programmatic stream serialization (the kernel may start while
 // the previous kernel on the stream finishes; it waits for it in griddep_wait) and, for

@@ -359,7 +359,7 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
                 __syncthreads();
             }
             if (active && nvalid > 0) {
-                T* q = out + ((size_t)y * W + x0) * a.dstride + (d_first - a.d_out0);
+                T* q = out + ((size_t)y * W + x0) * a.dstride + d_first;
 #pragma unroll
                 for (int i = 0; i < kL; ++i) {
                     if (x0 + i < W) *reinterpret_cast<unsigned*>(q) = fastdt_pack(v[i], ref[k * kCS + i], nvalid);
@@ -367,8 +367,9 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
                 }
             }
         } else if (active && nvalid > 0) {
-            // ---- store [H][W][dstride] ----
-            T* q = out + ((size_t)y * W + x0) * a.dstride + (d_first - a.d_out0);
+            // ---- store [slab][H][W][dstride] ----
+            T* q = out + (size_t)(d_first >> a.sd_shift) * a.slab_stride + ((size_t)y * W + x0) * a.dstride +
+                   (d_first & ((1 << a.sd_shift) - 1));
             if (vec && nvalid == 4 && x0 + kL <= W) {        // a whole chunk of whole groups
 #pragma unroll
                 for (int i = 0; i < kL; ++i) st4(q + (size_t)i * a.dstride, 4, true, v[i]);
