@@ -25,7 +25,7 @@ import threading
 from . import zncc as Z
 
 CANDIDATES = {
-    Z.ZNCC_TUNE_ROW_MINB2: [0, 1],
+    Z.ZNCC_TUNE_ROW_MINB2: [0, 1, 2],
     Z.ZNCC_TUNE_ROW_SPB: [0, 1, 2, 4, 8],
     Z.ZNCC_TUNE_H_TQ: [0, 2, 4, 8],
     Z.ZNCC_TUNE_V_TQ: [0, 2, 4, 8],

@@ -339,6 +339,21 @@ zncc_status run_coef(zncc_ctx* lc, const PairIO* io, int n, float sigma_s, float
     return ZNCC_OK;
 }
 
+// Lanes per 16-pixel chunk in the cost kernel: the warps of a row in 512 threads.
+int row_lanes(int W) { return W <= 1024 ? 8 : (W <= 2048 ? 4 : 2); }
+
+// Whether a context's cost kernel takes the two-blocks-per-SM variant (blocks of at most 320
+// threads): the second block hides the first one's latencies and barriers, but both stage the
+// rows that they visit, so it takes two units (row, slice) per block (us of the cost kernel with
+// one and two blocks: 640x192, D = 64, 1.3 units 29 and 31; 1242x375, D = 32, 2.5 units 49 and
+// 46; 1280x384, D = 128, 10 units 120 and 106; 600x1000, D = 40, 6.6 units 91 and 64). Not with
+// WTA alone, whose rows are whole units and whose running best spills there.
+bool row_two_blocks(const zncc_ctx* c, int mode) {
+    if (c->row_minb2) return c->row_minb2 == 1;
+    const int tq = row_lanes(c->W), nslices = (c->D + kG * tq - 1) / (kG * tq);
+    return mode != kModeWta && (long long)c->H * nslices >= 4ll * c->num_sms;
+}
+
 // Cost-kernel launches over the pairs (one per window radius among them). A block covers
 // one row and a run of disparity slices (the band of a block spans its slices, so the run
 // shrinks until the block fits in shared memory); in Wta mode a block covers every
@@ -348,12 +363,11 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
                      const char* what) {
     // pairs share a launch when they share the window radius and the block shape; a pair large
     // enough to fill the device by itself takes a launch of its own
-    auto tq_of = [](int W) { return W <= 1024 ? 8 : (W <= 2048 ? 4 : 2); };
     bool done[kMaxBatch] = {false};
     for (int first = 0; first < n; ++first) {
         if (done[first]) continue;
         const int r = io[first].c->r;
-        const int tq0 = tq_of(io[first].c->W), nch0 = padded_chunks(io[first].c->W, tq0);
+        const int tq0 = row_lanes(io[first].c->W), nch0 = padded_chunks(io[first].c->W, tq0);
         const bool alone = fills_device(io[first].c);
         RowBatch b;
         memset(&b, 0, sizeof(b));
@@ -361,9 +375,11 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
         b.fault = lc->fault;
         int threads = 0;
         size_t smem = 0;
-        bool minb2 = true;
+        // two blocks per SM where every pair of the launch allows it
+        bool minb2 = nch0 * tq0 <= 320;
+        for (int i = first; i < n; ++i) minb2 = minb2 && (done[i] || row_two_blocks(io[i].c, mode));
         for (int i = first; i < n; ++i) {
-            if (done[i] || io[i].c->r != r || tq_of(io[i].c->W) != tq0 || padded_chunks(io[i].c->W, tq0) != nch0 ||
+            if (done[i] || io[i].c->r != r || row_lanes(io[i].c->W) != tq0 || padded_chunks(io[i].c->W, tq0) != nch0 ||
                 (i != first && (alone || fills_device(io[i].c))))
                 continue;
             done[i] = true;
@@ -390,7 +406,7 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
             a.inv_sr255 = inv_sr255;
             a.coefH_out = mode == kModeHPair ? c->coefH : nullptr;
             a.s2 = s2;
-            a.minb2 = c->row_minb2;
+            a.minb2 = minb2 ? 1 : 0;
             a.wta.disp = io[i].disp;
             a.wta.first = 1;
             a.wta.last = 1;
@@ -406,12 +422,14 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
             // guide row's buffer fits in shared memory; else plain loads
             a.bulk = mode == kModeHPair && a.W % 16 == 0 && a.pitch % 16 == 0 &&
                      (uintptr_t)a.left % 16 == 0 && (uintptr_t)a.right % 16 == 0 && !c->row_nobulk ? 1 : 0;
-            while (!whole_rows && a.spb > 1 && zncc_row_smem_bytes(r, mode, dtype, a, nthr) > (size_t)lc->smem_max)
+            a.lpad = 1;
+            if (!minb2 && zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max) a.lpad = 0;
+            while (!whole_rows && a.spb > 1 && zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max)
                 --a.spb;
-            if (a.bulk && (zncc_row_smem_bytes(r, mode, dtype, a, nthr) > (size_t)lc->smem_max ||
-                           !zncc_row_bulk_fits_host(r, dtype, a, nthr)))
+            if (a.bulk && (zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max ||
+                           !zncc_row_bulk_fits_host(r, a)))
                 a.bulk = 0;
-            const size_t sm = zncc_row_smem_bytes(r, mode, dtype, a, nthr);
+            const size_t sm = zncc_row_layout(r, mode, dtype, a, nthr, minb2);
             if (sm > (size_t)lc->smem_max)
                 return fail(lc, ZNCC_EUNSUPPORTED, "the cost kernel's row band does not fit in shared memory");
             a.item0 = b.total_items;
@@ -419,7 +437,6 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
             b.total_items += a.nitems;
             threads = std::max(threads, nthr);
             smem = std::max(smem, sm);
-            minb2 = minb2 && a.minb2;
         }
         int bps = 0;
         const long long k0 = ((((long long)r * 4 + mode) * 4 + dtype) * 2 + (minb2 ? 1 : 0)) * 2 + (b.npairs == 1);
@@ -1120,7 +1137,7 @@ zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigm
     // the side kernels' blocks on every SM; its two-blocks-per-SM variant fills the registers,
     // so with the A_hat chain `reserve` SMs are left to it. FastDT needs A_hat_1 in the cost
     // kernel itself, so that pass comes first, on the main stream.
-    const int reserve = norm && lc->row_minb2 ? (lc->ahat_sms > 0 ? lc->ahat_sms : kAhatSideSms) : 0;
+    const int reserve = norm && lc->row_minb2 == 1 ? (lc->ahat_sms > 0 ? lc->ahat_sms : kAhatSideSms) : 0;
     int p_first_side = 1;
     if (dt == 2) {
         ZNCC_TRY(run_ahat(lc, io, n, 1, pfirst, npairs, K, inv_sr255, s2, true));
@@ -1743,7 +1760,10 @@ zncc_status zncc_set_tuning(zncc_ctx* c, int key, int value) {
     c->err.clear();
     if (value < 0) return fail(c, ZNCC_EINVAL, "tuning values are >= 0");
     switch (key) {
-        case ZNCC_TUNE_ROW_MINB2: c->row_minb2 = value ? 1 : 0; break;
+        case ZNCC_TUNE_ROW_MINB2:
+            if (value > 2) return fail(c, ZNCC_EINVAL, "blocks per SM of the cost kernel: 0, 1 (two) or 2 (one)");
+            c->row_minb2 = value;
+            break;
         case ZNCC_TUNE_ROW_SPB: c->row_spb = value; break;
         case ZNCC_TUNE_AHAT_SMS: c->ahat_sms = value; break;
         case ZNCC_TUNE_PLANE: c->plane_mode = value ? 1 : 0; break;

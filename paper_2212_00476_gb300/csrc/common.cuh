@@ -13,16 +13,41 @@ constexpr int kL = 16;
 constexpr int kG = 4;
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// Shared-memory arrays indexed by a pixel coordinate are stored as four interleaved
-// planes, entry idx at (idx & 3) * plane + (idx >> 2): in the access patterns below the
-// lanes of a warp share idx & 3 and spread over distinct idx >> 2, which keeps 16-byte
-// accesses free of bank conflicts (plain layouts put lanes 16 or 64 entries apart).
-__host__ __device__ __forceinline__ int plane_of(int len) { return ((len + 3) / 4 + 31) & ~31; }
-__device__ __forceinline__ int p4(int idx, int plane) { return (idx & 3) * plane + (idx >> 2); }
-// Entry start + i of a four-plane array, for start a multiple of 4 (i known at compile time).
-template <typename T>
-__device__ __forceinline__ T& at4(T* base, int start, int i, int plane) {
-    return base[(i & 3) * plane + (start >> 2) + (i >> 2)];
+// Shared-memory arrays of a cost row, indexed by a pixel coordinate and walked from a start that
+// is a multiple of 4 (16 chunk - 4 dq, or 12 t in the window statistics) with compile-time
+// steps: both layouts keep the lanes' 16-byte accesses in distinct banks, where a plain array would
+// put lanes 16 or 64 entries apart.
+//  - PAD: one spare entry after every four, entry idx at 5 * (idx >> 2) + (idx & 3). 5 (4 chunk -
+//    dq) takes every value mod 8, and mod 16 over half a warp. One pointer reaches every step at a
+//    constant offset, which is what fits beside the tile of sums in 96 registers.
+//  - else four interleaved planes, entry idx at (idx & 3) * plane + (idx >> 2): no spare entries,
+//    for rows whose padded bands would not fit.
+__host__ __device__ __forceinline__ int plane_of(int len) { return (len + 3) / 4; }
+template <bool PAD>
+__host__ __device__ __forceinline__ int cost_array_len(int len) {
+    return PAD ? (len + 3) / 4 * 5 : 4 * plane_of(len);
+}
+template <bool PAD, typename T>
+struct CostArray {
+    T* p;
+    int plane;                // (planes) entries between them
+    __device__ __forceinline__ T& operator[](int idx) const {
+        return PAD ? p[5 * (idx >> 2) + (idx & 3)] : p[(idx & 3) * plane + (idx >> 2)];
+    }
+    // the walk from entry `start`, a multiple of 4
+    __device__ __forceinline__ CostArray from(int start) const {
+        return CostArray{p + (PAD ? 5 * (start >> 2) : start >> 2), plane};
+    }
+    __device__ __forceinline__ T& at(int i) const {
+        return PAD ? p[5 * (i >> 2) + (i & 3)] : p[(i & 3) * plane + (i >> 2)];
+    }
+};
+// The thread's index, read anew: a value that the compiler does not keep in a register from an
+// earlier use.
+__device__ __forceinline__ int thread_index() {
+    int t;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+    return t;
 }
 // Per-position arrays of a DT line (coefficients, multipliers) are chunk-major: the kL entries of a chunk are contiguous and chunks are kCS = kL + 1 entries
 // apart. A thread then reaches every entry of its chunk at a constant offset from one
@@ -528,6 +553,131 @@ __device__ __forceinline__ void dt_pair(float (&v)[kL][4], const float4* __restr
                 fma4<PACKED>(b, G, v[i], v[i]);
             }
         }
+    }
+}
+
+// The same pass pair with the scan group given by the caller: the chunks' maps are composed in
+// groups of 2^scan_shift consecutive chunks (of one warp) by doubling rounds, then group by
+// group. The result depends on the groups in its last bits, not on the lanes per chunk
+// (LANES where known at compile time, else lanes). k: this thread's chunk of the line; sa / sb:
+// the line's scan buffers, 2 * nvg * lanes entries each, at this thread's lane of the chunk; bar:
+// the barrier of the line's bar_threads threads (0 with the whole block: the block's).
+template <bool SCALE, bool PACKED, int LANES, typename Hook, typename MulT>
+__device__ __forceinline__ void dt_group_pair(float (&v)[kL][4], const float4* __restrict__ co, int lanes_, int scan_shift, int lane,
+                                              int k, int nvg, float* sa, float4* sb, float s2,
+                                              const MulT* __restrict__ mul, int bar, int bar_threads,
+                                              Hook after_read) {
+    const int lanes = LANES ? LANES : lanes_;
+    const int scan = 1 << scan_shift, c = k & (scan - 1), vg = k >> scan_shift;     // place in the scan group, scan group
+    // ---- phase 1: forward sweep of the chunk with zero carry-in, scan of the group's maps ----
+    {
+        float u[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < kL; ++i) {
+            fma4<PACKED>(co[i].x, u, v[i], u);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[i][j] = u[j];
+        }
+    }
+    after_read();
+    float A = co[kL - 1].y, B[4], Ae, Be[4], F[4], G[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        B[j] = v[kL - 1][j];
+        F[j] = G[j] = 0.0f;
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int off = lanes << r;
+        if ((1 << r) >= scan) break;
+        const float A2 = __shfl_up_sync(kFull, A, off);
+        float B2[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) B2[j] = __shfl_up_sync(kFull, B[j], off);
+        if (c >= (1 << r)) {
+            fma4<PACKED>(A, B2, B, B);
+            A *= A2;
+        }
+    }
+    Ae = __shfl_up_sync(kFull, A, lanes);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) Be[j] = __shfl_up_sync(kFull, B[j], lanes);
+    if (c == 0) {
+        Ae = 1.0f;
+        Be[0] = Be[1] = Be[2] = Be[3] = 0.0f;
+    }
+    if (c == scan - 1) {
+        sa[vg * lanes] = A;
+        sb[vg * lanes] = make_float4(B[0], B[1], B[2], B[3]);
+    }
+    named_barrier(bar, bar_threads);
+
+    // ---- phase 2: carry from the groups before, corrected forward values, backward sweep ----
+#pragma unroll 1
+    for (int g = 0; g < vg; ++g) {
+        const float4 b2 = sb[g * lanes];
+        const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
+        fma4<PACKED>(sa[g * lanes], F, b4, F);
+    }
+    fma4<PACKED>(Ae, F, Be, F);
+    float h[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = kL - 1; i >= 0; --i) {
+        const float4 w = co[i];
+        float ft[4];
+        fma4<PACKED>(w.y, F, v[i], ft);
+        fma4<PACKED>(w.z, h, ft, h);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[i][j] = h[j];
+    }
+    A = co[0].w;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) B[j] = h[j];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int off = lanes << r;
+        if ((1 << r) >= scan) break;
+        const float A2 = __shfl_down_sync(kFull, A, off);
+        float B2[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) B2[j] = __shfl_down_sync(kFull, B[j], off);
+        if (c + (1 << r) < scan) {
+            fma4<PACKED>(A, B2, B, B);
+            A *= A2;
+        }
+    }
+    Ae = __shfl_down_sync(kFull, A, lanes);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) Be[j] = __shfl_down_sync(kFull, B[j], lanes);
+    if (c == scan - 1) {
+        Ae = 1.0f;
+        Be[0] = Be[1] = Be[2] = Be[3] = 0.0f;
+    }
+    float* sa2 = sa + nvg * lanes;
+    float4* sb2 = sb + nvg * lanes;
+    if (c == 0) {
+        sa2[vg * lanes] = A;
+        sb2[vg * lanes] = make_float4(B[0], B[1], B[2], B[3]);
+    }
+    named_barrier(bar, bar_threads);
+
+    // ---- phase 3: carry from the groups after, backward correction, scale ----
+#pragma unroll 1
+    for (int g = nvg - 1; g > vg; --g) {
+        const float4 b2 = sb2[g * lanes];
+        const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
+        fma4<PACKED>(sa2[g * lanes], G, b4, G);
+    }
+    fma4<PACKED>(Ae, G, Be, G);
+    if (SCALE && (mul || s2 != 1.0f)) {
+#pragma unroll
+        for (int i = 0; i < kL; ++i) {
+            fma4<PACKED>(co[i].w, G, v[i], v[i]);
+            mul4<PACKED>(mul ? out_scale(mul[i]) : s2, v[i]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kL; ++i) fma4<PACKED>(co[i].w, G, v[i], v[i]);
     }
 }
 

@@ -29,124 +29,6 @@ namespace zncc {
 // so that the copy is in flight during the whole step. A warp waits for its own chunks only
 // (an mbarrier per warp of a line), and the two barriers of the pass pair are per line: the
 // lines of a block share nothing but their boxes.
-template <bool SCALE, int lanes, typename Hook>
-__device__ __forceinline__ void dt_lines_pair(float (&v)[kL][4], const float4* __restrict__ co, int scan_shift, int lane,
-                                              int k, int nvg, float* sa, float4* sb, float s2,
-                                              const float2* __restrict__ mul, int bar, int bar_threads,
-                                              Hook after_read) {
-    const int scan = 1 << scan_shift, c = k & (scan - 1), vg = k >> scan_shift;     // place in the scan group, scan group
-    // ---- phase 1: forward sweep of the chunk with zero carry-in, scan of the group's maps ----
-    {
-        float u[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < kL; ++i) {
-            fma4<true>(co[i].x, u, v[i], u);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v[i][j] = u[j];
-        }
-    }
-    after_read();
-    float A = co[kL - 1].y, B[4], Ae, Be[4], F[4], G[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        B[j] = v[kL - 1][j];
-        F[j] = G[j] = 0.0f;
-    }
-#pragma unroll
-    for (int r = 0; (lanes << r) < 32; ++r) {
-        const int off = lanes << r;
-        if ((1 << r) >= scan) break;
-        const float A2 = __shfl_up_sync(kFull, A, off);
-        float B2[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) B2[j] = __shfl_up_sync(kFull, B[j], off);
-        if (c >= (1 << r)) {
-            fma4<true>(A, B2, B, B);
-            A *= A2;
-        }
-    }
-    Ae = __shfl_up_sync(kFull, A, lanes);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) Be[j] = __shfl_up_sync(kFull, B[j], lanes);
-    if (c == 0) {
-        Ae = 1.0f;
-        Be[0] = Be[1] = Be[2] = Be[3] = 0.0f;
-    }
-    if (c == scan - 1) {
-        sa[vg * lanes] = A;
-        sb[vg * lanes] = make_float4(B[0], B[1], B[2], B[3]);
-    }
-    named_barrier(bar, bar_threads);
-
-    // ---- phase 2: carry from the groups before, corrected forward values, backward sweep ----
-#pragma unroll 1
-    for (int g = 0; g < vg; ++g) {
-        const float4 b2 = sb[g * lanes];
-        const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
-        fma4<true>(sa[g * lanes], F, b4, F);
-    }
-    fma4<true>(Ae, F, Be, F);
-    float h[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int i = kL - 1; i >= 0; --i) {
-        const float4 w = co[i];
-        float ft[4];
-        fma4<true>(w.y, F, v[i], ft);
-        fma4<true>(w.z, h, ft, h);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[i][j] = h[j];
-    }
-    A = co[0].w;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) B[j] = h[j];
-#pragma unroll
-    for (int r = 0; (lanes << r) < 32; ++r) {
-        const int off = lanes << r;
-        if ((1 << r) >= scan) break;
-        const float A2 = __shfl_down_sync(kFull, A, off);
-        float B2[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) B2[j] = __shfl_down_sync(kFull, B[j], off);
-        if (c + (1 << r) < scan) {
-            fma4<true>(A, B2, B, B);
-            A *= A2;
-        }
-    }
-    Ae = __shfl_down_sync(kFull, A, lanes);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) Be[j] = __shfl_down_sync(kFull, B[j], lanes);
-    if (c == scan - 1) {
-        Ae = 1.0f;
-        Be[0] = Be[1] = Be[2] = Be[3] = 0.0f;
-    }
-    float* sa2 = sa + nvg * lanes;
-    float4* sb2 = sb + nvg * lanes;
-    if (c == 0) {
-        sa2[vg * lanes] = A;
-        sb2[vg * lanes] = make_float4(B[0], B[1], B[2], B[3]);
-    }
-    named_barrier(bar, bar_threads);
-
-    // ---- phase 3: carry from the groups after, backward correction, scale ----
-#pragma unroll 1
-    for (int g = nvg - 1; g > vg; --g) {
-        const float4 b2 = sb2[g * lanes];
-        const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
-        fma4<true>(sa2[g * lanes], G, b4, G);
-    }
-    fma4<true>(Ae, G, Be, G);
-    if (SCALE && (mul || s2 != 1.0f)) {
-#pragma unroll
-        for (int i = 0; i < kL; ++i) {
-            fma4<true>(co[i].w, G, v[i], v[i]);
-            mul4<true>(mul ? mul[i].y : s2, v[i]);
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < kL; ++i) fma4<true>(co[i].w, G, v[i], v[i]);
-    }
-}
-
 // The WTA of a step (Eq. (WTA1)): each thread takes the best of its four disparities at each
 // of its 16 positions, the chunk's lanes merge theirs by halving rounds (WtaRegs::merge), and
 // a lane keeps the running best of the 16 / lanes positions that it ends up with: a few
@@ -328,7 +210,7 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
 #pragma unroll
             for (int i = 0; i < kL; ++i) mul4<true>(mul[i].x, v[i]);
         }
-        dt_lines_pair<MODE != kLineWta, lanes>(v, co, b.s.scan_shift, lane, k, b.s.nvg, sa, sb, b.s2, mul, 1 + li, b.s.per_line,
+        dt_group_pair<MODE != kLineWta, true, lanes>(v, co, lanes, b.s.scan_shift, lane, k, b.s.nvg, sa, sb, b.s2, mul, 1 + li, b.s.per_line,
             [&]() {
                 // the box has been read: the lines' warps say so, and its loader refills it
                 __syncwarp();

@@ -1044,13 +1044,12 @@ cudaError_t launch_wta_volume(const void* cost, int dtype, int W, int H, int D, 
     return cudaGetLastError();
 }
 
-bool zncc_row_bulk_fits_host(int R, int dtype, const RowArgs& a, int nthreads) {
-    return zncc_row_bulk_fits(R, dtype, a, nthreads);
+bool zncc_row_bulk_fits_host(int R, const RowArgs& a) { return zncc_row_bulk_fits(R, a); }
+
+size_t zncc_row_layout(int R, int mode, int dtype, RowArgs& a, int nthreads, bool minb2) {
+    return zncc_row_fill_layout(R, mode, dtype, a, nthreads, minb2);
 }
 
-size_t zncc_row_smem_bytes(int R, int mode, int dtype, const RowArgs& a, int nthreads) {
-    return zncc_row_smem(R, mode, dtype, a, nthreads);
-}
 
 cudaError_t launch_zncc_row(int R, const RowBatch& b, int threads, size_t smem, int mode, int dtype,
                             cudaStream_t st) {

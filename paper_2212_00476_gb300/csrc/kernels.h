@@ -37,10 +37,15 @@ struct RowArgs {
     const float2* mulmap;     // (HPair, FastDT codes) [H][W]: (unused, output scale (1-K)^2/A_hat_1)
     float s2;                 // (1 - K)^2
     WtaOut wta;               // (Wta)
-    int minb2;                // use the two-blocks-per-SM variant where the block allows
+    int minb2;                // use the two-blocks-per-SM variant (blocks of at most 320 threads)
     int bulk;                 // (HPair) stage the image rows by bulk asynchronous copies: both
                               // images and the pitch 16-byte aligned, W a multiple of 16
     int item0, nitems;        // this pair's units (row, slice), or rows (Wta), in a batched launch
+    int lpad;                 // spare entries (0, or 1 with minb2) per chunk of the left band and statistics
+    // filled by zncc_row_layout: log2(tq), the planes of the cost arrays, and byte offsets in shared memory of the packed right
+    // band, the window statistics, the coefficients, the scan buffers, FastDT's output scales and
+    // references, and the guide row (bulk)
+    int tq_shift, rp_plane, sr_plane, rp_off, sl_off, sr_off, co_off, sb_off, sa_off, mrow_off, ref_off, grow_off;
 };
 
 // One cost-kernel launch over up to kMaxBatch pairs of the same window radius, passed by
@@ -163,14 +168,15 @@ cudaError_t launch_dt_lines_f16(const DtBatch<kMaxBatch>& b, size_t smem, int mo
 void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, dim3 grid, dim3 block, size_t smem,
                    cudaStream_t st, int cluster);
 
-size_t zncc_row_smem_bytes(int R, int mode, int dtype, const RowArgs& a, int nthreads);
+// Completes the arguments' shared-memory layout; returns the dynamic shared memory of a block.
+size_t zncc_row_layout(int R, int mode, int dtype, RowArgs& a, int nthreads, bool minb2);
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) for a kernel on the current device, made only
 // when the size exceeds what an earlier call set (a launch pays for it once, not every time);
 // forget_smem_attributes() drops the record (zncc_create calls it, so that contexts created
 // after a device reset set the attributes again).
 cudaError_t set_max_smem(const void* fn, size_t smem);
 void forget_smem_attributes();
-bool zncc_row_bulk_fits_host(int R, int dtype, const RowArgs& a, int nthreads);
+bool zncc_row_bulk_fits_host(int R, const RowArgs& a);
 // A pass whose coefficients (and multipliers) can be streamed (at least two slices per line
 // group); the shared memory of a block with one or two buffers of them.
 bool line_coef_async(const LineArgs& a);

@@ -16,6 +16,11 @@ namespace zncc {
 // d0 + 4dq + 3 of each slice. The chunk count is padded to whole warps; pixels x >= W are
 // computed from clamped reads and dropped.
 //
+// Bound by the latency of its phases (window sums, normalisation, the pass pair and its two
+// barriers a slice) and by shared-memory wavefronts, not by its store of the volume (38 us at
+// 1280x384x128 F32): the 96-register variant with two blocks per SM (20 warps) takes 104-106 us
+// there at 48% of the issue slots, one block with 128 registers 117-119 us at 42%.
+//
 // Cost (Eq. (1) through Eq. (2)): with P = sum over the window of I_R(x+i, y+j) *
 // I_T(x-d+i, y+j), n = (2R+1)^2 and the window sums S of each image,
 //   C = (n P - S_R(x) S_T(x-d)) * inv_sigma_R(x) * inv_sigma_T(x-d),
@@ -66,8 +71,8 @@ __device__ __forceinline__ void pack4_raw(const uint8_t* raw, int Wr, int xs, ui
     for (int c = 0; c < 4; ++c) col[c] = make_uint4(o[c][0], o[c][1], o[c][2], o[c][3]);
 }
 
-// Centres per item of the window statistics. An item's column walk reads up to kStatsItem - 1
-// columns past the last centre of the band, so the packed band planes hold kStatsItem spare
+// Centres per run of the right window statistics. A run's column walk reads up to kStatsItem - 1
+// columns past the last centre of the band, so the packed right band holds kStatsItem spare
 // entries.
 constexpr int kStatsItem = 12;
 
@@ -75,9 +80,9 @@ constexpr int kStatsItem = 12;
 __host__ __device__ inline int bulk_row_stride(int W) { return W + 16; }
 
 // One visit of the cost kernel: row y of one pair, disparity slices [s_begin, s_end).
-// Threads beyond the pair's nch * tq (whole warps) only take part in the barriers. Returns
+// The block has the pair's nch * tq threads. Returns
 // false when a bulk copy of the image rows timed out (the fault is recorded; the block stops).
-template <int R, typename T, int MODE>
+template <int R, typename T, int MODE, bool PAD>
 __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_begin, int s_end,
                                               uint4* smem_u4, unsigned long long* bar, unsigned& phase,
                                               unsigned* fault) {
@@ -87,32 +92,34 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
     const int W = a.W, H = a.H;
     const int tid = threadIdx.x;
     const int nthr = nch * tq;
-    const bool active = tid < nthr;
-    const int k = active ? tid / tq : 0, dq = active ? tid - (tid / tq) * tq : 0;
-    const int lane = tid & 31, wl = tid >> 5, nwl = nthr >> 5;
     // every lane's disparities lie in [blk_lo, blk_hi)
     const int blk_lo = a.d_lo + s_begin * ds, blk_hi = a.d_lo + s_end * ds;
 
-    // ---- shared memory carve ----
+    // ---- shared memory carve (zncc_row_layout) ----
     const int NLP = span + 2 * R;                      // left columns x' in [-R, span+R)
     const int NRP = span + 2 * R + (blk_hi - blk_lo) - 1;
     const int xr0 = -R - (blk_hi - 1);                 // right columns x'' in [xr0, xr0+NRP)
     const int NSR = span + (blk_hi - blk_lo) - 1;      // right centres c in [c0, c0+NSR)
     const int c0 = -(blk_hi - 1);
-    const int pLP = plane_of(NLP + kStatsItem), pRP = plane_of(NRP + kStatsItem), pX = plane_of(span), pSR = plane_of(NSR);
-    uint4* LP = smem_u4;
-    uint4* RP = LP + 4 * pLP;
-    int2* SL = reinterpret_cast<int2*>(RP + 4 * pRP);               // (S, 1/sigma bits) per x
-    int2* SR = SL + 4 * pX;                                          // per right centre
-    float4* co = reinterpret_cast<float4*>(SR + 4 * pSR);            // HPair, chunk-major
-    float4* sb = co + nch * kCS;
-    float* sa = reinterpret_cast<float*>(sb + 2 * nwl * tq);
+    unsigned char* const sm = reinterpret_cast<unsigned char*>(smem_u4);
+    // The left columns and statistics are chunk-major (entry 0 = column -R resp. x = 0): the
+    // lanes of a chunk read the same entry and the eight chunks of a warp distinct banks, one
+    // shared-memory wavefront a load where a layout with two chunks to a bank group takes four.
+    // (lpad: the spare entry per chunk, left out where the row would not fit with it.)
+    uint4* const LP = smem_u4;
+    const int lpad = PAD ? 1 : a.lpad;
+    auto lpos = [&](int idx) { return idx + (idx >> 4) * lpad; };
+    const CostArray<PAD, uint4> RP{reinterpret_cast<uint4*>(sm + a.rp_off), a.rp_plane};
+    // (S, 1/sigma bits) per x, and per right centre
+    int2* const SL = reinterpret_cast<int2*>(sm + a.sl_off);
+    const CostArray<PAD, int2> SR{reinterpret_cast<int2*>(sm + a.sr_off), a.sr_plane};
+    float4* const co = reinterpret_cast<float4*>(sm + a.co_off);     // HPair, chunk-major
     // FastDT codes (HPair): the row's output scales and the reference values v(d_arb = 0)
     constexpr bool kFast = std::is_same<T, uint8_t>::value;
-    float* mrow = sa + 2 * nwl * tq;                                 // chunk-major (kCS)
-    float* ref = mrow + nch * kCS;
-    // (bulk) the guide row y for the coefficients, after everything else
-    uint8_t* grow = reinterpret_cast<uint8_t*>(kFast ? ref + nch * kCS : mrow);
+    float* const mrow = reinterpret_cast<float*>(sm + a.mrow_off);   // chunk-major (kCS)
+    float* const ref = reinterpret_cast<float*>(sm + a.ref_off);
+    // (bulk) the guide row y for the coefficients
+    uint8_t* const grow = sm + a.grow_off;
 
     // ---- stage the packed bands (and the DT coefficients) ----
     const bool bulk = MODE == kModeHPair && a.bulk;
@@ -121,7 +128,7 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
         // region that the statistics and coefficients take once the bands are packed, and of
         // the guide row y; one thread issues them, every thread waits on the mbarrier.
         const int Wr = bulk_row_stride(W);
-        uint8_t* rawL = reinterpret_cast<uint8_t*>(SL);
+        uint8_t* rawL = sm + a.sl_off;
         uint8_t* rawR = rawL + l * Wr;
         fence_proxy_async_smem();                       // earlier accesses of the region, then the copies
         __syncthreads();
@@ -158,19 +165,23 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
             const int g4 = left ? g : g - ngl;
             const int xs = left ? 4 * g4 - R : xr0 + 4 * g4;   // image column of entry 4 g4
             const int nent = left ? NLP : NRP;
-            uint4* dst = left ? LP : RP;
-            const int pl = left ? pLP : pRP;
+            const CostArray<PAD, uint4> rdst = RP.from(4 * g4);
+            uint4* const ldst = LP + lpos(4 * g4);
+            auto put = [&](int c, const uint4& col) {
+                if (left) ldst[c] = col;
+                else rdst.at(c) = col;
+            };
             const uint8_t* raw = left ? rawL : rawR;
             if (xs >= 0 && xs + 3 < W && 4 * g4 + 3 < nent) {
                 uint4 col[4];
                 if (left) pack4_raw<l, SLS>(raw, Wr, xs, col);
                 else pack4_raw<l, SRS>(raw, Wr, xs, col);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) dst[c * pl + g4] = col[c];
+                for (int c = 0; c < 4; ++c) put(c, col[c]);
             } else {
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    if (4 * g4 + c < nent) dst[c * pl + g4] = pack1(raw, min(max(xs + c, 0), W - 1));
+                    if (4 * g4 + c < nent) put(c, pack1(raw, min(max(xs + c, 0), W - 1)));
             }
         }
         __syncthreads();                                 // the raw rows are consumed
@@ -184,8 +195,8 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
             for (int j = 0; j < l; ++j) w[j >> 2] |= (unsigned)img[roff[j] + xc] << (8 * (j & 3));
             return make_uint4(w[0], w[1], w[2], w[3]);
         };
-        for (int t = tid; t < NLP; t += blockDim.x) LP[p4(t, pLP)] = pack(a.left, min(max(t - R, 0), W - 1));
-        for (int t = tid; t < NRP; t += blockDim.x) RP[p4(t, pRP)] = pack(a.right, min(max(xr0 + t, 0), W - 1));
+        for (int t = tid; t < NLP; t += blockDim.x) LP[lpos(t)] = pack(a.left, min(max(t - R, 0), W - 1));
+        for (int t = tid; t < NRP; t += blockDim.x) RP[t] = pack(a.right, min(max(xr0 + t, 0), W - 1));
     }
     if constexpr (MODE == kModeHPair) {
         // the row's DT coefficients (w, chunk prefix product, next w, chunk suffix product),
@@ -216,82 +227,85 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
     }
     __syncthreads();
 
-    // ---- window statistics: kSC consecutive centres per thread, left then right ----
-    // Items of 12 centres start 12 columns apart, so the 16-byte column loads of the eight
-    // lanes of a quarter warp fall in distinct bank groups (16 apart, they would share two).
-    constexpr int kSC = kStatsItem;
+    // ---- window statistics: runs of consecutive centres per thread, left then right ----
+    // Left runs are chunks; right runs start 12 columns apart, so that the 16-byte column loads of
+    // the eight lanes of a quarter warp fall in distinct bank groups (16 apart, they would share
+    // two).
     const unsigned n = (unsigned)(l * l);
     // A fused horizontal pair (F32, F16) in the scaled form multiplies its result by
     // s2 = (1-K)^2; the pair is linear, so the factor rides on the left 1/sigma instead
     // (FastDT codes take per-position scales in the pair).
     const float lscale = (MODE == kModeHPair && !kFast) ? a.s2 : 1.0f;
-    const int nlc = (span + kSC - 1) / kSC, nrc = (NSR + kSC - 1) / kSC;
-    for (int t = tid; t < nlc + nrc; t += blockDim.x) {
-        const bool is_left = t < nlc;
-        const int cs = is_left ? t * kSC : c0 + (t - nlc) * kSC;   // first centre
-        const uint4* col = is_left ? LP : RP;
-        const int pc = is_left ? pLP : pRP;
-        const int ib = is_left ? cs : cs - R - xr0;                 // column index of cs - R
-        // (ib = 12 t, or 12 (t - nlc) on the right: both multiples of 4)
-        int Sx[kSC], Qx[kSC];
-#pragma unroll
-        for (int i = 0; i < kSC; ++i) Sx[i] = Qx[i] = 0;
+    // the statistics of COUNT centres whose first window starts at column 0 of the walk
+    auto stats = [&](auto count, auto column, auto store) {
+        constexpr int COUNT = decltype(count)::value;
+        int Sx[COUNT], Qx[COUNT];           // (an entry lives from its first touch to its centre's store)
         unsigned ps = 0u, pq = 0u;
 #pragma unroll
-        for (int u = 0; u < kSC + 2 * R; ++u) {
-            const uint4 w = at4(col, ib, u, pc);
+        for (int u = 0; u < COUNT + 2 * R; ++u) {
+            const uint4 w = column(u);
             ps = __dp4a(w.x, 0x01010101u, ps);
             pq = __dp4a(w.x, w.x, pq);
             if (NW > 1) { ps = __dp4a(w.y, 0x01010101u, ps); pq = __dp4a(w.y, w.y, pq); }
             if (NW > 2) { ps = __dp4a(w.z, 0x01010101u, ps); pq = __dp4a(w.z, w.z, pq); }
             if (NW > 3) { ps = __dp4a(w.w, 0x01010101u, ps); pq = __dp4a(w.w, w.w, pq); }
-            if (u - 2 * R >= 0 && u - 2 * R < kSC) { Sx[u - 2 * R] += (int)ps; Qx[u - 2 * R] += (int)pq; }
-            if (u + 1 < kSC) { Sx[u + 1] -= (int)ps; Qx[u + 1] -= (int)pq; }
-        }
-#pragma unroll
-        for (int i = 0; i < kSC; ++i) {
-            const int var = (int)(n * (unsigned)Qx[i] - (unsigned)Sx[i] * (unsigned)Sx[i]);
-            const float is = var > 0 ? rsqrtf((float)var) : 0.0f;      // as k_window_stats
-            const int2 st = make_int2(Sx[i], __float_as_int(is_left ? is * lscale : is));
-            if (is_left) {
-                if (cs + i < span) at4(SL, cs, i, pX) = st;
-            } else if (cs + i - c0 < NSR) {
-                at4(SR, cs - c0, i, pSR) = st;
+            if (u + 1 < COUNT) { Sx[u + 1] = (int)ps; Qx[u + 1] = (int)pq; }
+            const int i = u - 2 * R;                                    // the centre completed
+            if (i >= 0 && i < COUNT) {
+                const int S = (int)ps - (i > 0 ? Sx[i] : 0), Q = (int)pq - (i > 0 ? Qx[i] : 0);
+                const int var = (int)(n * (unsigned)Q - (unsigned)S * (unsigned)S);
+                store(i, S, var > 0 ? rsqrtf((float)var) : 0.0f);          // as k_window_stats
             }
+        }
+    };
+    const int nrc = (NSR + kStatsItem - 1) / kStatsItem;
+    for (int t = tid; t < nch + nrc; t += blockDim.x) {
+        if (t < nch) {
+            const uint4* const col = LP + lpos(t * kL);
+            int2* const out = SL + lpos(t * kL);
+            stats(std::integral_constant<int, kL>(), [&](int u) { return col[u + (u >> 4) * lpad]; },
+                  [&](int i, int S, float is) { out[i] = make_int2(S, __float_as_int(is * lscale)); });
+        } else {
+            const int c = (t - nch) * kStatsItem;                       // first centre, from c0
+            const CostArray<PAD, uint4> col = RP.from(c);               // (its first column is c0 + c - R = xr0 + c)
+            const CostArray<PAD, int2> out = SR.from(c);
+            stats(std::integral_constant<int, kStatsItem>(), [&](int u) { return col.at(u); },
+                  [&](int i, int S, float is) { if (c + i < NSR) out.at(i) = make_int2(S, __float_as_int(is)); });
         }
     }
     __syncthreads();
 
-    const int x0 = k * kL;
-    T* out = reinterpret_cast<T*>(a.vol);
     const bool vec = a.vec != 0;
     WtaRegs wr;
     if constexpr (MODE == kModeWta) wr.reset();
 
     for (int sl = s_begin; sl < s_end; ++sl) {
-        const int d_first = a.d_lo + sl * ds + dq * kG;
-        const int nvalid = max(0, min(4, a.d_hi - d_first));
         float v[kL][4];
-        if (active) {
+        // A thread's place (chunk, lane of the chunk) is taken from its index anew in each phase:
+        // the tile of sums leaves few registers for what would be kept across it.
+        {
+            const int t1 = thread_index(), x0 = (t1 >> a.tq_shift) * kL;
+            const int d_first = a.d_lo + sl * ds + (t1 & (tq - 1)) * kG;
             // ---- window sums of products, times n, for 16 pixels x 4 disparities ----
             // n P[i] = n prefix(i + 2R) - n prefix(i - 1): each entry is set at its first touch
             // (-n prefix(i - 1) at step i - 1; n P[0] at step 2R) and completed at step i + 2R;
             // the factor n of Eq. (2)'s numerator rides on those multiply-adds (mod 2^32)
             unsigned P[kL][4];
-            // RP index of column x' - d_first - j at step t (x' = x0 - R + t) is rbase + t - j;
-            // rbase + 1 = x0 - d_first + blk_hi is a multiple of 4 (as are x0, d_first and
-            // blk_hi, d_lo being one), so every index below has a constant plane
-            const int rbase = x0 - R - d_first - xr0;      // >= 3: d_first + 3 < blk_hi
-            const int rb4 = rbase + 1;
+            // RP index of column x' - d_first - j at step t (x' = x0 - R + t) is rbase + t - j,
+            // rbase = x0 - R - d_first - xr0 >= 3 (d_first + 3 < blk_hi); rbase + 1 = x0 - d_first +
+            // blk_hi is a multiple of 4 (as are x0, d_first and blk_hi, d_lo being one), so the
+            // columns are at constant offsets from the pointer to entry rbase + 1 - 4
+            const uint4* const lpp = LP + lpos(x0);
+            const CostArray<PAD, uint4> rpp = RP.from(x0 - d_first + blk_hi - 4);
             uint4 rp[4];
-            rp[1] = at4(RP, rb4, -2, pRP);
-            rp[2] = at4(RP, rb4, -3, pRP);
-            rp[3] = at4(RP, rb4, -4, pRP);
+            rp[1] = rpp.at(2);
+            rp[2] = rpp.at(1);
+            rp[3] = rpp.at(0);
             unsigned pre[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
             for (int t = 0; t < kL + 2 * R; ++t) {
-                const uint4 lp = at4(LP, x0, t, pLP);
-                rp[0] = at4(RP, rb4, t - 1, pRP);
+                const uint4 lp = lpp[t + (t >> 4) * lpad];
+                rp[0] = rpp.at(t + 3);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     pre[j] = __dp4a(lp.x, rp[j].x, pre[j]);
@@ -308,68 +322,69 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
             }
 
             // ---- normalization, Eq. (2); the target statistics slide like the columns ----
-            const int cb = x0 - d_first - c0;               // SR index of (i, j) is cb + i - j >= 3
-            const int cb4 = cb + 1;                         // a multiple of 4, like rb4
+            // (SR index of (i, j) is x0 - d_first - c0 + i - j >= 3, one less than a multiple of 4)
+            const int t2 = thread_index(), xn = (t2 >> a.tq_shift) * kL;
+            const int dn = a.d_lo + sl * ds + (t2 & (tq - 1)) * kG;
+            const int2* const slp = SL + lpos(xn);
+            const CostArray<PAD, int2> srp = SR.from(xn - dn + blk_hi - 4);
             int2 sr[4];
-            sr[1] = at4(SR, cb4, -2, pSR);
-            sr[2] = at4(SR, cb4, -3, pSR);
-            sr[3] = at4(SR, cb4, -4, pSR);
-            auto normalize = [&](auto full) {
+            sr[1] = srp.at(2);
+            sr[2] = srp.at(1);
+            sr[3] = srp.at(0);
+            // Pixels past the row and disparities past the range are computed like the others (their
+            // columns and statistics are staged) and never stored or compared; the zero weights
+            // past the row keep them out of the pass pair.
 #pragma unroll
-                for (int i = 0; i < kL; ++i) {
-                    const int x = x0 + i;
-                    const int2 st = at4(SL, x0, i, pX);
-                    sr[0] = at4(SR, cb4, i - 1, pSR);
-                    const float isl = __int_as_float(st.y);      // (times the pair's scale)
-                    const unsigned nsl = 0u - (unsigned)st.x;
+            for (int i = 0; i < kL; ++i) {
+                const int2 st = slp[i];
+                sr[0] = srp.at(i + 3);
+                const float isl = __int_as_float(st.y);      // (times the pair's scale)
+                const unsigned nsl = 0u - (unsigned)st.x;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const unsigned num = nsl * (unsigned)sr[j].x + P[i][j];       // n P - S_R S_T
-                        const float c = (float)(int)num * isl * __int_as_float(sr[j].y);
-                        if constexpr (decltype(full)::value) v[i][j] = c;
-                        else v[i][j] = (x < W && j < nvalid) ? c : 0.0f;
-                    }
-                    sr[3] = sr[2];
-                    sr[2] = sr[1];
-                    sr[1] = sr[0];
+                for (int j = 0; j < 4; ++j) {
+                    const unsigned num = nsl * (unsigned)sr[j].x + P[i][j];       // n P - S_R S_T
+                    v[i][j] = (float)(int)num * isl * __int_as_float(sr[j].y);
                 }
-            };
-            // whole chunks of whole 4-disparity groups take the path without predicates
-            if (x0 + kL <= W && nvalid == 4) normalize(std::true_type());
-            else normalize(std::false_type());
+                sr[3] = sr[2];
+                sr[2] = sr[1];
+                sr[1] = sr[0];
+            }
         }
 
         if constexpr (MODE == kModeWta) {
-            if (active) wr.fold(v, nvalid, d_first);
+            const int t3 = thread_index(), dn = a.d_lo + sl * ds + (t3 & (tq - 1)) * kG;
+            wr.fold(v, max(0, min(4, a.d_hi - dn)), dn);
             continue;
         }
-        if constexpr (MODE == kModeHPair && kFast)
-            dt_pair(v, co + k * kCS, tq, dq, lane, wl, nwl, sa, sb, a.s2, mrow + k * kCS, NoHook(), active);
-        else if constexpr (MODE == kModeHPair)       // s2 already folded into the costs
-            dt_pair<false>(v, co + k * kCS, tq, dq, lane, wl, nwl, sa, sb, 1.0f, (const float2*)nullptr,
-                           NoHook(), active);
-
+        const int t3 = thread_index(), k = t3 >> a.tq_shift, dq = t3 & (tq - 1);
+        if constexpr (MODE == kModeHPair) {
+            float4* const sb = reinterpret_cast<float4*>(sm + a.sb_off);
+            float* const sa = reinterpret_cast<float*>(sm + a.sa_off);
+            const int shift = 5 - a.tq_shift, nvg = nthr >> 5;      // scan groups: the warps
+            dt_group_pair<kFast, PAD, 0>(v, co + k * kCS, tq, shift, t3 & 31, k, nvg, sa + dq, sb + dq, kFast ? a.s2 : 1.0f,
+                                          kFast ? mrow + k * kCS : (const float*)nullptr, 0, nthr, NoHook());
+        }
+        const int x0 = k * kL, d_first = a.d_lo + sl * ds + dq * kG;
+        const int nvalid = max(0, min(4, a.d_hi - d_first));
+        T* q = reinterpret_cast<T*>(a.vol) + (size_t)(d_first >> a.sd_shift) * a.slab_stride +
+               ((size_t)y * W + x0) * a.dstride + (d_first & ((1 << a.sd_shift) - 1));    // [slab][H][W][dstride]
         if constexpr (kFast) {
             // near-zero-mean codes against d_arb = 0, held by lane dq 0 in slice 0 (a visit covers
             // every slice of its row, in order)
             if (sl == 0) {
-                if (dq == 0 && active)
+                if (dq == 0)
 #pragma unroll
                     for (int i = 0; i < kL; ++i) ref[k * kCS + i] = v[i][0];
                 __syncthreads();
             }
-            if (active && nvalid > 0) {
-                T* q = out + ((size_t)y * W + x0) * a.dstride + d_first;
+            if (nvalid > 0) {
 #pragma unroll
                 for (int i = 0; i < kL; ++i) {
                     if (x0 + i < W) *reinterpret_cast<unsigned*>(q) = fastdt_pack(v[i], ref[k * kCS + i], nvalid);
                     q += a.dstride;
                 }
             }
-        } else if (active && nvalid > 0) {
-            // ---- store [slab][H][W][dstride] ----
-            T* q = out + (size_t)(d_first >> a.sd_shift) * a.slab_stride + ((size_t)y * W + x0) * a.dstride +
-                   (d_first & ((1 << a.sd_shift) - 1));
+        } else if (nvalid > 0) {
             if (vec && nvalid == 4 && x0 + kL <= W) {        // a whole chunk of whole groups
 #pragma unroll
                 for (int i = 0; i < kL; ++i) st4(q + (size_t)i * a.dstride, 4, true, v[i]);
@@ -384,10 +399,10 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
     }
 
     if constexpr (MODE == kModeWta) {
-        if (active) {
+        {
             // the chunk's lanes merge their running bests; each lane writes its share of positions
-            wr.merge(tq, lane, [&](int i, float best, int bd) {
-                const int x = x0 + i;
+            wr.merge(tq, tid & 31, [&](int i, float best, int bd) {
+                const int x = (tid >> a.tq_shift) * kL + i;
                 if (x < W) {
                     const size_t o = (size_t)y * W + x;
                     if (!a.wta.first) {                                // earlier launches: smaller d
@@ -445,35 +460,45 @@ __global__ void __launch_bounds__(MINB == 2 ? 320 : 512, MINB) k_zncc_row(const 
             u += s_end - s_begin;
         }
         if (u >= i1) griddep_launch_dependents();       // this block's last visit
-        if (!zncc_row_item<R, T, MODE>(a, y, s_begin, s_end, smem_u4, &bar, phase, b.fault)) return;
+        if (!zncc_row_item<R, T, MODE, MINB == 2>(a, y, s_begin, s_end, smem_u4, &bar, phase, b.fault)) return;
         __syncthreads();                                 // the next visit restages shared memory
     }
 }
 
-// Shared-memory bytes of one item of k_zncc_row.
-inline size_t zncc_row_smem(int R, int mode, int dtype, const RowArgs& a, int nthreads) {
+// The shared memory of a visit of k_zncc_row: offsets into a, bytes returned. pad: for the
+// two-blocks-per-SM variant (CostArray).
+inline size_t zncc_row_fill_layout(int R, int mode, int dtype, RowArgs& a, int nthreads, bool pad) {
     const int ds = kG * a.tq, span = a.nch * kL;
     const int nslices = (a.d_hi - a.d_lo + ds - 1) / ds;
     const int drange = std::min(a.spb, nslices) * ds;
-    size_t b = 16ull * 4 * (plane_of(span + 2 * R + kStatsItem) + plane_of(span + 2 * R + drange - 1 + kStatsItem));
-    const int pX = plane_of(span);
-    b += 8ull * 4 * (pX + plane_of(span + drange - 1));
-    if (mode == kModeHPair) b += 16ull * a.nch * kCS + dt_scan_bytes(nthreads / 32, a.tq);
-    if (mode == kModeHPair && dtype == 2) b += 8ull * a.nch * kCS;       // FastDT: scales, references
-    if (mode == kModeHPair && a.bulk) b += (size_t)(a.W + 15) / 16 * 16; // the guide row
-    return b;
+    a.tq_shift = 0;
+    while ((1 << a.tq_shift) < a.tq) ++a.tq_shift;
+    auto len = [&](int n) { return pad ? cost_array_len<true>(n) : cost_array_len<false>(n); };
+    const int nlp = span + 2 * R, nrp = nlp + drange - 1 + kStatsItem, nsr = span + drange - 1;
+    a.rp_plane = plane_of(nrp);
+    a.sr_plane = plane_of(nsr);
+    int b = 16 * (kL + a.lpad) * ((nlp + kL - 1) / kL);
+    auto take = [&](int& off, int bytes) {
+        off = b = (b + 15) & ~15;
+        b += bytes;
+    };
+    const bool pair = mode == kModeHPair, fast = pair && dtype == 2;
+    take(a.rp_off, 16 * len(nrp));
+    take(a.sl_off, 8 * (kL + a.lpad) * a.nch);
+    take(a.sr_off, 8 * len(nsr));
+    take(a.co_off, pair ? 16 * a.nch * kCS : 0);
+    take(a.sb_off, pair ? 2 * (nthreads / 32) * a.tq * 16 : 0);
+    take(a.sa_off, pair ? 2 * (nthreads / 32) * a.tq * 4 : 0);
+    take(a.mrow_off, fast ? 4 * a.nch * kCS : 0);
+    take(a.ref_off, fast ? 4 * a.nch * kCS : 0);
+    take(a.grow_off, pair && a.bulk ? (a.W + 15) / 16 * 16 : 0);
+    return (size_t)b;
 }
 
 // Whether a visit's raw rows (both images, bulk_row_stride apart) fit in the shared memory that
 // the statistics and the later per-visit arrays take (HPair): the region after the packed bands.
-inline bool zncc_row_bulk_fits(int R, int dtype, const RowArgs& a, int nthreads) {
-    const int ds = kG * a.tq, span = a.nch * kL;
-    const int nslices = (a.d_hi - a.d_lo + ds - 1) / ds;
-    const int drange = std::min(a.spb, nslices) * ds;
-    size_t after = 8ull * 4 * (plane_of(span) + plane_of(span + drange - 1)) + 16ull * a.nch * kCS +
-                   dt_scan_bytes(nthreads / 32, a.tq);
-    if (dtype == 2) after += 8ull * a.nch * kCS;
-    return 2ull * (2 * R + 1) * bulk_row_stride(a.W) <= after;
+inline bool zncc_row_bulk_fits(int R, const RowArgs& a) {
+    return 2 * (2 * R + 1) * bulk_row_stride(a.W) <= a.grow_off - a.sl_off;
 }
 
 template <int R, int MINB, bool SINGLE>
@@ -501,7 +526,7 @@ static void (*row_fn(int mode, int dtype, bool minb2, bool single))(RowBatch) {
 template <int R>
 cudaError_t zncc_row_occupancy_impl(int mode, int dtype, int threads, size_t smem, bool minb2, bool single,
                                     int* bps) {
-    void (*fn)(RowBatch) = row_fn<R>(mode, dtype, minb2 && threads <= 320, single);
+    void (*fn)(RowBatch) = row_fn<R>(mode, dtype, minb2, single);
     if (!fn) return cudaErrorInvalidValue;
     cudaError_t e = set_max_smem((const void*)fn, smem);
     if (e != cudaSuccess) return e;
@@ -511,9 +536,7 @@ cudaError_t zncc_row_occupancy_impl(int mode, int dtype, int threads, size_t sme
 template <int R>
 cudaError_t launch_zncc_row_impl(const RowBatch& b, int threads, size_t smem, int mode, int dtype,
                                  cudaStream_t st) {
-    bool minb2 = true;
-    for (int i = 0; i < b.npairs; ++i) minb2 = minb2 && b.p[i].minb2;
-    void (*fn)(RowBatch) = row_fn<R>(mode, dtype, minb2 && threads <= 320, b.npairs == 1);
+    void (*fn)(RowBatch) = row_fn<R>(mode, dtype, b.p[0].minb2 != 0, b.npairs == 1);
     if (!fn) return cudaErrorInvalidValue;
     cudaError_t e = set_max_smem((const void*)fn, smem);
     if (e != cudaSuccess) return e;
