@@ -412,10 +412,10 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
             a.wta.last = 1;
             const int nthr = a.nch * a.tq;
             const int nslices = (c->D + kG * a.tq - 1) / (kG * a.tq);
-            // WTA keeps a row's running best in registers, FastDT codes each slice against the
-            // row's d = 0: a block then visits whole rows
-            const bool whole_rows = mode == kModeWta || dtype == 2;
-            if (whole_rows) a.spb = nslices;
+            // WTA keeps a row's running best in registers: a block then visits whole rows. FastDT codes
+            // need slice 0 of the row in every visit, so a visit takes all the slices it can.
+            const bool whole_rows = mode == kModeWta;
+            if (whole_rows || dtype == 2) a.spb = nslices;
             else a.spb = c->row_spb > 0 ? std::min(c->row_spb, nslices) : nslices;
             // the image rows by bulk copies where both images and the pitch are 16-byte aligned
             // and W is a multiple of 16, while the rows fit in the region they share and the
@@ -424,7 +424,7 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
                      (uintptr_t)a.left % 16 == 0 && (uintptr_t)a.right % 16 == 0 && !c->row_nobulk ? 1 : 0;
             a.lpad = 1;
             if (!minb2 && zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max) a.lpad = 0;
-            while (!whole_rows && a.spb > 1 && zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max)
+            while (!whole_rows && dtype != 2 && a.spb > 1 && zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max)
                 --a.spb;
             if (a.bulk && (zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max ||
                            !zncc_row_bulk_fits_host(r, a)))
@@ -898,9 +898,28 @@ zncc_status run_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* passe
         b.stage_bytes = (long long)stage;
         b.fault = lc->fault;
         b.drill = lc->wait_drill;
-        const size_t smem = stage + rest;
+        size_t smem = stage + rest;
         if (smem > (size_t)lc->smem_max) return fail(lc, ZNCC_EUNSUPPORTED, "DT pass exceeds shared memory");
         ZNCC_CUDA(lc, size_line_grid(b, threads, smem, mode, dtype, lc->num_sms, lc), "occupancy query");
+        if (dtype == 2 && mode == kLineStore && b.co_async && a0.cs == 1) {
+            // FastDT stores go by whole line groups, so the last round leaves blocks idle: with one
+            // coefficient buffer more blocks may fit and the groups take fewer block rounds per SM
+            // (rows of 1280x384: 384 groups in two rounds of 2 blocks per SM, or one of 3)
+            const int two = b.grid;
+            size_t rest1 = 0;
+            for (int i = 0; i < b.npairs; ++i)
+                rest1 = std::max(rest1, line_pair_smem_bytes(mode, dtype, b.p[i], false) - line_stage_bytes(dtype, b.p[i]));
+            ZNCC_CUDA(lc, size_line_grid(b, threads, stage + rest1, mode, dtype, lc->num_sms, lc), "occupancy query");
+            auto block_rounds = [&](int grid) {
+                return (long long)((b.total_items + grid - 1) / grid) * ((grid + lc->num_sms - 1) / lc->num_sms);
+            };
+            if (block_rounds(b.grid) < block_rounds(two)) {
+                b.co_async = 0;
+                smem = stage + rest1;
+            } else {
+                b.grid = two;
+            }
+        }
         ZNCC_LAUNCH(lc, kind, launch_line_batch(b, threads, smem, mode, dtype, lc->cur), "DT pass pair");
     }
     return ZNCC_OK;

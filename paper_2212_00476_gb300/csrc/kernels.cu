@@ -807,10 +807,16 @@ __global__ void __launch_bounds__(512) k_line_pair(const __grid_constant__ LineB
             }
             T* q = vol + (line_ok ? elem0(a, o) : 0);
             const long long es = a.elem_stride;
+            if (any && npos >= kL && nvalid == 4) {              // a whole chunk of whole groups
 #pragma unroll
-            for (int i = 0; i < kL; ++i)
-                if (any && i < npos)
-                    *reinterpret_cast<unsigned*>(q + (size_t)i * es) = fastdt_pack(v[i], ref_all[cthr + i], nvalid);
+                for (int i = 0; i < kL; ++i)
+                    *reinterpret_cast<unsigned*>(q + (size_t)i * es) = fastdt_pack(v[i], ref_all[cthr + i], 4);
+            } else if (any) {
+#pragma unroll
+                for (int i = 0; i < kL; ++i)
+                    if (i < npos)
+                        *reinterpret_cast<unsigned*>(q + (size_t)i * es) = fastdt_pack(v[i], ref_all[cthr + i], nvalid);
+            }
         } else {
             T* q = vol + (line_ok ? elem0(a, o) : 0);
             const long long es = a.elem_stride;

@@ -92,8 +92,12 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
     const int W = a.W, H = a.H;
     const int tid = threadIdx.x;
     const int nthr = nch * tq;
+    // FastDT codes are against d_arb = 0: a visit that starts past slice 0 computes that slice
+    // first, for its references alone
+    constexpr bool kFast = std::is_same<T, uint8_t>::value;
+    const int s_first = kFast ? 0 : s_begin;
     // every lane's disparities lie in [blk_lo, blk_hi)
-    const int blk_lo = a.d_lo + s_begin * ds, blk_hi = a.d_lo + s_end * ds;
+    const int blk_lo = a.d_lo + s_first * ds, blk_hi = a.d_lo + s_end * ds;
 
     // ---- shared memory carve (zncc_row_layout) ----
     const int NLP = span + 2 * R;                      // left columns x' in [-R, span+R)
@@ -115,7 +119,6 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
     const CostArray<PAD, int2> SR{reinterpret_cast<int2*>(sm + a.sr_off), a.sr_plane};
     float4* const co = reinterpret_cast<float4*>(sm + a.co_off);     // HPair, chunk-major
     // FastDT codes (HPair): the row's output scales and the reference values v(d_arb = 0)
-    constexpr bool kFast = std::is_same<T, uint8_t>::value;
     float* const mrow = reinterpret_cast<float*>(sm + a.mrow_off);   // chunk-major (kCS)
     float* const ref = reinterpret_cast<float*>(sm + a.ref_off);
     // (bulk) the guide row y for the coefficients
@@ -279,7 +282,7 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
     WtaRegs wr;
     if constexpr (MODE == kModeWta) wr.reset();
 
-    for (int sl = s_begin; sl < s_end; ++sl) {
+    for (int sl = s_first; sl < s_end; sl = kFast && sl < s_begin ? s_begin : sl + 1) {
         float v[kL][4];
         // A thread's place (chunk, lane of the chunk) is taken from its index anew in each phase:
         // the tile of sums leaves few registers for what would be kept across it.
@@ -369,15 +372,19 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
         T* q = reinterpret_cast<T*>(a.vol) + (size_t)(d_first >> a.sd_shift) * a.slab_stride +
                ((size_t)y * W + x0) * a.dstride + (d_first & ((1 << a.sd_shift) - 1));    // [slab][H][W][dstride]
         if constexpr (kFast) {
-            // near-zero-mean codes against d_arb = 0, held by lane dq 0 in slice 0 (a visit covers
-            // every slice of its row, in order)
+            // near-zero-mean codes against d_arb = 0, held by lane dq 0 in slice 0, the visit's first
             if (sl == 0) {
                 if (dq == 0)
 #pragma unroll
                     for (int i = 0; i < kL; ++i) ref[k * kCS + i] = v[i][0];
                 __syncthreads();
             }
-            if (nvalid > 0) {
+            if (sl < s_begin) {                              // (stored by the visit that owns slice 0)
+            } else if (nvalid == 4 && x0 + kL <= W) {        // a whole chunk of whole groups
+#pragma unroll
+                for (int i = 0; i < kL; ++i)
+                    *reinterpret_cast<unsigned*>(q + (size_t)i * a.dstride) = fastdt_pack(v[i], ref[k * kCS + i], 4);
+            } else if (nvalid > 0) {
 #pragma unroll
                 for (int i = 0; i < kL; ++i) {
                     if (x0 + i < W) *reinterpret_cast<unsigned*>(q) = fastdt_pack(v[i], ref[k * kCS + i], nvalid);
@@ -424,8 +431,7 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
 // SINGLE: the launch holds one pair, whose arguments are then read at constant offsets of
 // the parameter block instead of through a dynamic index.
 // Work units: (row, disparity slice) in row-major order, pair by pair (Wta: whole rows, since
-// a row's running best stays in registers; FastDT codes: whole rows, since every slice is
-// coded against d = 0 of the first). Block b takes the units [b*total/G, (b+1)*total/G)
+// a row's running best stays in registers). Block b takes the units [b*total/G, (b+1)*total/G)
 // and visits them row by row, at most spb slices per visit, so that the band of a row is
 // staged once per visit and every block gets the same work within one unit.
 template <int R, typename T, int MODE, int MINB, bool SINGLE>
@@ -447,7 +453,7 @@ __global__ void __launch_bounds__(MINB == 2 ? 320 : 512, MINB) k_zncc_row(const 
         const int nslices = (a.d_hi - a.d_lo + ds - 1) / ds;
         const int local = u - a.item0;
         int y, s_begin, s_end;
-        if constexpr (MODE == kModeWta || std::is_same<T, uint8_t>::value) {     // whole rows
+        if constexpr (MODE == kModeWta) {       // whole rows
             y = local;
             s_begin = 0;
             s_end = nslices;
