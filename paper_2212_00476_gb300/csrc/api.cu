@@ -315,13 +315,14 @@ struct PairIO {
 // DT coefficients of every pair (guide = left image), one launch.
 zncc_status run_coef(zncc_ctx* lc, const PairIO* io, int n, float sigma_s, float sigma_r, bool rows = true) {
     CoefBatch b;
-    memset(&b, 0, sizeof(b));
+    static_cast<CoefHead&>(b) = CoefHead{};
     b.npairs = n;
     const float K = (float)exp(-1.0 / (double)sigma_s);
     const float inv = (float)(1.0 / (255.0 * (double)sigma_r));
     long long t = 0;
     for (int i = 0; i < n; ++i) {
         CoefArgs& a = b.p[i];
+        a = CoefArgs{};
         a.guide = io[i].left;
         a.pitch = io[i].pitch;
         a.W = io[i].c->W;
@@ -370,7 +371,7 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
         const int tq0 = row_lanes(io[first].c->W), nch0 = padded_chunks(io[first].c->W, tq0);
         const bool alone = fills_device(io[first].c);
         RowBatch b;
-        memset(&b, 0, sizeof(b));
+        static_cast<RowHead&>(b) = RowHead{};
         b.mode = mode;
         b.fault = lc->fault;
         int threads = 0;
@@ -385,6 +386,7 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
             done[i] = true;
             zncc_ctx* c = io[i].c;
             RowArgs& a = b.p[b.npairs++];
+            a = RowArgs{};
             a.left = io[i].left;
             a.right = io[i].right;
             a.pitch = io[i].pitch;
@@ -787,6 +789,7 @@ zncc_status run_dt_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* pa
             const int W = c->W, H = c->H;
             b.tmap[b.npairs] = tmaps[i];
             DtArgs& a = b.p[b.npairs++];
+            a = DtArgs{};
             a.vol = p.vol;
             a.pos_stride = p.horiz ? p.dstride : (long long)W * p.dstride;
             a.line_stride = p.horiz ? (long long)W * p.dstride : p.dstride;
@@ -883,7 +886,7 @@ zncc_status run_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* passe
         const LineArgs& a0 = args[first];
         const bool alone = fills_device(ctxs[first]);
         LineBatch b;
-        memset(&b, 0, sizeof(b));
+        static_cast<LineHead&>(b) = LineHead{};
         int threads = 0;
         size_t stage = 0, rest = 0;
         for (int i = first; i < n; ++i) {
@@ -956,7 +959,7 @@ constexpr int kAhatSideSms = 8;
 zncc_status run_ahat(zncc_ctx* lc, const PairIO* io, int n, int p, int pfirst, int npairs, float K,
                      float inv_sr255, float s2, bool fast) {
     AhatBatch b;
-    memset(&b, 0, sizeof(b));
+    static_cast<AhatHead&>(b) = AhatHead{};
     b.npairs = n;
     b.horiz = (p % 2) == 1;
     b.K = K;
@@ -969,6 +972,7 @@ zncc_status run_ahat(zncc_ctx* lc, const PairIO* io, int n, int p, int pfirst, i
         zncc_ctx* c = io[i].c;
         const size_t npix = (size_t)c->W * c->H;
         AhatArgs& a = b.p[i];
+        a = AhatArgs{};
         a.guide = io[i].left;
         a.pitch = io[i].pitch;
         a.W = c->W;
@@ -1074,7 +1078,7 @@ zncc_status run_plane(zncc_ctx* lc, const PairIO* io, int n, float sigma_s, floa
         ZNCC_LAUNCH(lc, K_PLANE, launch_plane(b, cls, smem, lc->cur), "plane-resident ZNCC + DT + WTA");
     }
     WtaFinishBatch fb;
-    memset(&fb, 0, sizeof(fb));
+    static_cast<WtaFinishHead&>(fb) = WtaFinishHead{};
     fb.npairs = n;
     for (int i = 0; i < n; ++i) {
         fb.p[i].keys = io[i].c->keys;
@@ -1236,7 +1240,7 @@ zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigm
         ZNCC_TRY(run_lines(lc, ctxs, lp, n, kind));
     }
     WtaFinishBatch fb;                              // keys -> disparities, keys zeroed
-    memset(&fb, 0, sizeof(fb));
+    static_cast<WtaFinishHead&>(fb) = WtaFinishHead{};
     fb.npairs = n;
     for (int i = 0; i < n; ++i) {
         fb.p[i].keys = io[i].c->keys;
@@ -1534,9 +1538,10 @@ zncc_status dt_aggregate_noalloc(const uint8_t* guide, int pitch, int width, int
     float4* coefV = coefH + npix;
 
     CoefBatch cb;
-    memset(&cb, 0, sizeof(cb));
+    static_cast<CoefHead&>(cb) = CoefHead{};
     cb.npairs = 1;
     CoefArgs& ca = cb.p[0];
+    ca = CoefArgs{};
     ca.guide = guide;
     ca.pitch = pitch;
     ca.W = width;
@@ -1562,7 +1567,7 @@ zncc_status dt_aggregate_noalloc(const uint8_t* guide, int pitch, int width, int
         fill_line_args(a, lp, width, height, coefH, coefV);
         ZNCC_TRY(noalloc_plan(*d, a, lp));
         LineBatch b;
-        memset(&b, 0, sizeof(b));
+        static_cast<LineHead&>(b) = LineHead{};
         int threads = 0;
         size_t stage = 0, rest = 0;
         add_line_pair(b, a, kLineStore, dtype, threads, stage, rest);

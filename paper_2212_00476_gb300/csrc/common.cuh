@@ -135,7 +135,7 @@ __device__ __forceinline__ void st4(__half* p, int nvalid, bool vec, const float
 // word, the lowest disparity in the lowest byte. The passes that code and decode every element
 // are bound by these instructions, so both work on pairs of values in the halves of a word:
 // about 11 instructions an element to code and 5 to decode, where one value at a time took 16
-// and 7 (1280x384x128: V pair @I8V@, H pair @I8H@ us).
+// and 7 (1280x384x128: V pair 163 -> 121 us, H pair 289 -> 169).
 constexpr float kFastT = 16383.0f;
 
 // Bytes picked by the nibbles of s; a nibble with its top bit set gives the picked byte's sign

@@ -310,24 +310,15 @@ cudaError_t DT_NAME(launch_dt_lines)(const DtBatch<kMaxBatch>& b, size_t smem, i
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config(cfg, attr, dim3(b.grid), dim3(threads), smem, st, 1);
-    if (b.npairs == 1) {                    // one pair: a small parameter block, read at constant offsets
-        DtBatch<1> o;
-        o.npairs = 1;
-        o.total_steps = b.total_steps;
-        o.grid = b.grid;
-        o.drill = b.drill;
-        o.s2 = b.s2;
-        o.fault = b.fault;
-        o.s = b.s;
-        o.p[0] = b.p[0];
-        o.tmap[0] = b.tmap[0];
-        void (*fn)(DtBatch<1>) = dt_lines_fn<1>(mode, b.s.lanes, threads);
-        cudaError_t e = set_max_smem((const void*)fn, smem);
-        return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, fn, o);
-    }
-    void (*fn)(DtBatch<kMaxBatch>) = dt_lines_fn<kMaxBatch>(mode, b.s.lanes, threads);
-    cudaError_t e = set_max_smem((const void*)fn, smem);
-    return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, fn, b);
+    const bool single = b.npairs == 1;
+    const void* fn = single ? (const void*)dt_lines_fn<1>(mode, b.s.lanes, threads)
+                            : (const void*)dt_lines_fn<kMaxBatch>(mode, b.s.lanes, threads);
+    cudaError_t e = set_max_smem(fn, smem);
+    if (e != cudaSuccess) return e;
+    if (!single) return launch_batch(cfg, fn, b);
+    DtBatch<1> o = first_pair<DtHead>(b);
+    o.tmap[0] = b.tmap[0];
+    return launch_batch(cfg, fn, o);
 }
 
 }  // namespace zncc

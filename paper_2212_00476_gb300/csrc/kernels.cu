@@ -219,12 +219,13 @@ cudaError_t launch_window_stats(const uint8_t* img, int pitch, int W, int H, int
 //   (w(p), prod_{j=c..p} w(j), w(p+1), prod_{j=p..c+15} w(j+1)),  c = chunk start (16 | c).
 // coefH is [H][W]; coefV is [W][H] (a column is contiguous). One thread per position; the
 // 16 positions of a chunk are 16 consecutive lanes, whose products are shuffle scans.
-__global__ void k_dt_coef(const __grid_constant__ CoefBatch b) {
+template <int NP>
+__global__ void k_dt_coef(const __grid_constant__ CoefBatchOf<NP> b) {
     griddep_wait();
     const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     int pi = 0;
-    while (pi + 1 < b.npairs && gid >= b.p[pi + 1].thread0) ++pi;
-    const CoefArgs& a = b.p[pi];
+    while (NP > 1 && pi + 1 < b.npairs && gid >= b.p[pi + 1].thread0) ++pi;
+    const CoefArgs& a = b.p[NP > 1 ? pi : 0];
     const int W = a.W, H = a.H;
     const int nchH = (W + kL - 1) / kL, nchV = (H + kL - 1) / kL;
     const long long local = gid - a.thread0;
@@ -271,15 +272,16 @@ __global__ void k_dt_coef(const __grid_constant__ CoefBatch b) {
 constexpr int kAhatWarps = 4;
 constexpr int kAhatArrays = 3;      // per line: weights, inputs, values
 
-__global__ void __launch_bounds__(32 * kAhatWarps) k_ahat_pair(const __grid_constant__ AhatBatch b) {
+template <int NP>
+__global__ void __launch_bounds__(32 * kAhatWarps) k_ahat_pair(const __grid_constant__ AhatBatchOf<NP> b) {
     extern __shared__ float ahat_smem[];
     griddep_wait();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int gline = blockIdx.x * kAhatWarps + wib;
     if (gline >= b.total_lines) return;
     int pi = 0;
-    while (pi + 1 < b.npairs && gline >= b.p[pi + 1].line0) ++pi;
-    const AhatArgs& a = b.p[pi];
+    while (NP > 1 && pi + 1 < b.npairs && gline >= b.p[pi + 1].line0) ++pi;
+    const AhatArgs& a = b.p[NP > 1 ? pi : 0];
     const int line = gline - a.line0;
     const bool horiz = b.horiz != 0;
     const int W = a.W, n = horiz ? a.W : a.H;
@@ -376,12 +378,14 @@ size_t ahat_pass_smem_bytes(int nmax) { return (size_t)kAhatWarps * kAhatArrays 
 
 cudaError_t launch_ahat_pair(const AhatBatch& b, cudaStream_t st) {
     const size_t smem = ahat_pass_smem_bytes(b.nmax);
-    cudaError_t e = set_max_smem((const void*)k_ahat_pair, smem);
+    cudaError_t e = b.npairs == 1 ? set_max_smem((const void*)k_ahat_pair<1>, smem)
+                                  : set_max_smem((const void*)k_ahat_pair<kMaxBatch>, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config(cfg, attr, dim3((b.total_lines + kAhatWarps - 1) / kAhatWarps), dim3(32 * kAhatWarps), smem, st, 1);
-    return cudaLaunchKernelEx(&cfg, k_ahat_pair, b);
+    return b.npairs == 1 ? launch_batch(cfg, (const void*)k_ahat_pair<1>, first_pair<AhatHead>(b))
+                         : launch_batch(cfg, (const void*)k_ahat_pair<kMaxBatch>, b);
 }
 
 // The column coefficients alone (coefV), coalesced: thread (column x, chunk c) computes the
@@ -390,13 +394,14 @@ cudaError_t launch_ahat_pair(const AhatBatch& b, cudaStream_t st) {
 // each column's 256 contiguous bytes go out together. Values as in k_dt_coef.
 constexpr int kColWarps = 4;
 
-__global__ void __launch_bounds__(32 * kColWarps) k_dt_coef_cols(const __grid_constant__ CoefBatch b) {
+template <int NP>
+__global__ void __launch_bounds__(32 * kColWarps) k_dt_coef_cols(const __grid_constant__ CoefBatchOf<NP> b) {
     __shared__ float4 tile[kColWarps][32][kL + 1];
     griddep_wait();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     int pi = 0;
-    while (pi + 1 < b.npairs && (long long)blockIdx.x >= b.p[pi + 1].thread0) ++pi;
-    const CoefArgs& a = b.p[pi];
+    while (NP > 1 && pi + 1 < b.npairs && (long long)blockIdx.x >= b.p[pi + 1].thread0) ++pi;
+    const CoefArgs& a = b.p[NP > 1 ? pi : 0];
     const int W = a.W, H = a.H;
     const int nchV = (H + kL - 1) / kL, ncg = (nchV + kColWarps - 1) / kColWarps;
     const int local = (int)(blockIdx.x - a.thread0);
@@ -443,7 +448,8 @@ cudaError_t launch_dt_coef_cols(const CoefBatch& b, cudaStream_t st) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config(cfg, attr, dim3((unsigned)b.total_threads), dim3(32 * kColWarps), 0, st, 1);
-    return cudaLaunchKernelEx(&cfg, k_dt_coef_cols, b);
+    return b.npairs == 1 ? launch_batch(cfg, (const void*)k_dt_coef_cols<1>, first_pair<CoefHead>(b))
+                         : launch_batch(cfg, (const void*)k_dt_coef_cols<kMaxBatch>, b);
 }
 
 long long dt_coef_threads(int W, int H) {
@@ -455,7 +461,8 @@ cudaError_t launch_dt_coef(const CoefBatch& b, cudaStream_t st) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config(cfg, attr, dim3((unsigned)blocks), dim3(256), 0, st, 1);
-    return cudaLaunchKernelEx(&cfg, k_dt_coef, b);
+    return b.npairs == 1 ? launch_batch(cfg, (const void*)k_dt_coef<1>, first_pair<CoefHead>(b))
+                         : launch_batch(cfg, (const void*)k_dt_coef<kMaxBatch>, b);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -490,7 +497,7 @@ size_t line_stage_bytes(int dtype, const LineArgs& a) {
 // pairs. SINGLE: the launch holds one pair, whose arguments are then all read at constant
 // offsets instead of through a dynamic index. CLUSTER: lines span the CTAs of a cluster.
 template <typename T, int MODE, bool SINGLE, bool CLUSTER>
-__global__ void __launch_bounds__(512) k_line_pair(const __grid_constant__ LineBatch b) {
+__global__ void __launch_bounds__(512) k_line_pair(const __grid_constant__ LineBatchOf<SINGLE ? 1 : kMaxBatch> b) {
     extern __shared__ __align__(128) float4 smem4[];
     // (tma) per staging buffer and warp, an mbarrier that the first lanes of the warp's chunks
     // arrive on once per fill (a line is whole warps, so a chunk never straddles two warps)
@@ -893,33 +900,33 @@ cudaError_t launch_fastdt_codec(const int16_t* values, int n, uint8_t* codes, in
 }
 
 template <bool SINGLE, bool CLUSTER>
-static void (*line_pair_fn_t(int mode, int dtype))(LineBatch) {
+static const void* line_pair_fn_t(int mode, int dtype) {
     if (mode == kLineStore)
-        return dtype == 0 ? k_line_pair<float, kLineStore, SINGLE, CLUSTER>
-                          : dtype == 1 ? k_line_pair<__half, kLineStore, SINGLE, CLUSTER>
-                                       : k_line_pair<uint8_t, kLineStore, SINGLE, CLUSTER>;
-    return dtype == 0 ? k_line_pair<float, kLineWta, SINGLE, CLUSTER>
-                      : dtype == 1 ? k_line_pair<__half, kLineWta, SINGLE, CLUSTER>
-                                   : k_line_pair<uint8_t, kLineWta, SINGLE, CLUSTER>;
+        return dtype == 0   ? (const void*)k_line_pair<float, kLineStore, SINGLE, CLUSTER>
+               : dtype == 1 ? (const void*)k_line_pair<__half, kLineStore, SINGLE, CLUSTER>
+                            : (const void*)k_line_pair<uint8_t, kLineStore, SINGLE, CLUSTER>;
+    return dtype == 0   ? (const void*)k_line_pair<float, kLineWta, SINGLE, CLUSTER>
+           : dtype == 1 ? (const void*)k_line_pair<__half, kLineWta, SINGLE, CLUSTER>
+                        : (const void*)k_line_pair<uint8_t, kLineWta, SINGLE, CLUSTER>;
 }
 
-static void (*line_pair_fn(int mode, int dtype, bool single, bool cluster))(LineBatch) {
+static const void* line_pair_fn(int mode, int dtype, bool single, bool cluster) {
     if (cluster) return single ? line_pair_fn_t<true, true>(mode, dtype) : line_pair_fn_t<false, true>(mode, dtype);
     return single ? line_pair_fn_t<true, false>(mode, dtype) : line_pair_fn_t<false, false>(mode, dtype);
 }
 
 cudaError_t line_pair_occupancy(int mode, int dtype, int threads, size_t smem, bool single, bool cluster,
                                 int* blocks_per_sm) {
-    void (*fn)(LineBatch) = line_pair_fn(mode, dtype, single, cluster);
-    cudaError_t e = set_max_smem((const void*)fn, smem);
+    const void* fn = line_pair_fn(mode, dtype, single, cluster);
+    cudaError_t e = set_max_smem(fn, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
 }
 
 cudaError_t line_pair_max_clusters(int mode, int dtype, int threads, size_t smem, bool single, int cs,
                                    int* clusters) {
-    void (*fn)(LineBatch) = line_pair_fn(mode, dtype, single, true);
-    cudaError_t e = set_max_smem((const void*)fn, smem);
+    const void* fn = line_pair_fn(mode, dtype, single, true);
+    cudaError_t e = set_max_smem(fn, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs);
@@ -938,23 +945,27 @@ cudaError_t line_pair_max_clusters(int mode, int dtype, int threads, size_t smem
 cudaError_t launch_line_batch(const LineBatch& b, int threads, size_t smem, int mode, int dtype,
                               cudaStream_t st) {
     const int cs = b.p[0].cs;
-    void (*fn)(LineBatch) = line_pair_fn(mode, dtype, b.npairs == 1, cs > 1);
-    cudaError_t e = set_max_smem((const void*)fn, smem);
+    const void* fn = line_pair_fn(mode, dtype, b.npairs == 1, cs > 1);
+    cudaError_t e = set_max_smem(fn, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config(cfg, attr, dim3(b.grid), dim3(threads), smem, st, cs);
-    return cudaLaunchKernelEx(&cfg, fn, b);
+    if (b.npairs > 1) return launch_batch(cfg, fn, b);
+    LineBatchOf<1> o = first_pair<LineHead>(b);
+    o.tmap[0] = b.tmap[0];
+    return launch_batch(cfg, fn, o);
 }
 
 // ---------------------------------------------------------------------------------------
 // End of the fused WTA: key -> disparity, key -> 0 (ready for the next run).
-__global__ void k_wta_finish(const __grid_constant__ WtaFinishBatch b) {
+template <int NP>
+__global__ void k_wta_finish(const __grid_constant__ WtaFinishBatchOf<NP> b) {
     griddep_wait();
     const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     int pi = 0;
-    while (pi + 1 < b.npairs && gid >= b.p[pi + 1].thread0) ++pi;
-    const WtaFinishArgs& a = b.p[pi];
+    while (NP > 1 && pi + 1 < b.npairs && gid >= b.p[pi + 1].thread0) ++pi;
+    const WtaFinishArgs& a = b.p[NP > 1 ? pi : 0];
     const long long i = gid - a.thread0;
     if (i < a.npix) {
         a.disp[i] = wta_key_disparity(a.keys[i]);
@@ -967,7 +978,8 @@ cudaError_t launch_wta_finish(const WtaFinishBatch& b, cudaStream_t st) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config(cfg, attr, dim3((unsigned)blocks), dim3(256), 0, st, 1);
-    return cudaLaunchKernelEx(&cfg, k_wta_finish, b);
+    return b.npairs == 1 ? launch_batch(cfg, (const void*)k_wta_finish<1>, first_pair<WtaFinishHead>(b))
+                         : launch_batch(cfg, (const void*)k_wta_finish<kMaxBatch>, b);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -50,11 +50,18 @@ struct RowArgs {
 
 // One cost-kernel launch over up to kMaxBatch pairs of the same window radius, passed by
 // value. Of G blocks, block b takes the units [b * total / G, (b+1) * total / G), in order.
-struct RowBatch {
+// A launch of one pair passes the same head with that pair alone: a parameter block of a few
+// hundred bytes, read at constant offsets, where the full one is several thousand that every
+// launch copies (a cost volume of 160x64, D = 16: 6.0 -> 5.5 us a call).
+struct RowHead {
     int npairs, total_items, grid, mode;
     unsigned* fault;          // device word of the launching context: bits of kFault* set by the kernel
-    RowArgs p[kMaxBatch];
 };
+template <int NP>
+struct RowBatchOf : RowHead {
+    RowArgs p[NP];
+};
+using RowBatch = RowBatchOf<kMaxBatch>;
 
 // Device-side faults a kernel records instead of waiting without end (ZNCC_FAULT_* of zncc.h).
 constexpr unsigned kFaultBulkWait = 1u;      // a bulk copy of image rows did not complete in time
@@ -104,17 +111,29 @@ struct LineArgs {
 // block b takes the items [b * total / G, (b+1) * total / G) of all pairs, in order; an item is
 // one step (line group, disparity slice) in both modes, or a whole line group for FastDT
 // stores.
-struct LineBatch {
+struct LineHead {
     int npairs, total_items, total_steps, grid;
     int co_async;             // coefficients streamed by cp.async (two buffers; line_coef_async)
     long long stage_bytes;    // staging region (the largest pair's), before the other arrays
     unsigned* fault;          // device fault word (kFaultTmaWait), or NULL without TMA
     int drill;                // (tests) one thread per block waits out an mbarrier nobody arrives on
-    LineArgs p[kMaxBatch];
+};
+template <int NP>
+struct LineBatchOf : LineHead {
+    LineArgs p[NP];
     // (tma) per pair: the input volume as a 3-D tensor {entries per pixel, W, H}, box
     // {4 tq, 16, 1} (rows) or {4 tq, 1, 16} (columns): one chunk's positions of one slice
-    CUtensorMap tmap[kMaxBatch];
+    CUtensorMap tmap[NP];
 };
+using LineBatch = LineBatchOf<kMaxBatch>;
+// The launch of one pair alone: the head and the first pair of a batch.
+template <typename Head, template <int> class Batch>
+Batch<1> first_pair(const Batch<kMaxBatch>& b) {
+    Batch<1> o;
+    static_cast<Head&>(o) = b;
+    o.p[0] = b.p[0];
+    return o;
+}
 
 // The DT pass pair over a volume stored in slabs of sd = 2^sd_shift disparities, [slab][H][W][sd]
 // (one slab of all disparities: a caller's [H][W][D] volume): dt_lines.cu.
@@ -145,12 +164,14 @@ struct DtShape {
     // coefficient array, and byte offsets in shared memory
     int scan_shift, mul, per_line, nwl, nvg, slot, ps, line_off, arr, co_off, mul_off, scan_off;
 };
-template <int NP>
-struct DtBatch {
+struct DtHead {
     int npairs, total_steps, grid, drill;
     float s2;
     unsigned* fault;
     DtShape s;
+};
+template <int NP>
+struct DtBatch : DtHead {
     DtArgs p[NP];
     CUtensorMap tmap[NP];     // {sd, W, H, slabs}, box {4 lanes, lines, 16, 1} (columns) or {4 lanes, 16, lines, 1}
 };
@@ -167,6 +188,11 @@ cudaError_t launch_dt_lines_f16(const DtBatch<kMaxBatch>& b, size_t smem, int mo
 // cluster > 1, thread-block clusters of that many CTAs along x. attr must hold 2 entries.
 void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, dim3 grid, dim3 block, size_t smem,
                    cudaStream_t st, int cluster);
+template <typename Batch>
+cudaError_t launch_batch(const cudaLaunchConfig_t& cfg, const void* fn, const Batch& b) {
+    void* args[] = {const_cast<Batch*>(&b)};
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
 
 // Completes the arguments' shared-memory layout; returns the dynamic shared memory of a block.
 size_t zncc_row_layout(int R, int mode, int dtype, RowArgs& a, int nthreads, bool minb2);
@@ -219,11 +245,15 @@ struct CoefArgs {
     float4* coefV;            // [W][H]
     long long thread0;        // first thread (k_dt_coef_cols: block) of this pair in the launch
 };
-struct CoefBatch {
+struct CoefHead {
     int npairs;
     long long total_threads;
-    CoefArgs p[kMaxBatch];
 };
+template <int NP>
+struct CoefBatchOf : CoefHead {
+    CoefArgs p[NP];
+};
+using CoefBatch = CoefBatchOf<kMaxBatch>;
 cudaError_t launch_dt_coef(const CoefBatch& b, cudaStream_t st);
 
 // One DT pass pair over an A_hat plane (the response of an all-ones plane, Sec. IV-C), a
@@ -238,12 +268,16 @@ struct AhatArgs {
     int in_mul;               // mulmap.x = ain (1) or 1 (0)
     int line0;                // first line of this pair in the launch
 };
-struct AhatBatch {
+struct AhatHead {
     int npairs, total_lines, horiz, nmax;
     float K, inv_sr255, s2;
     float xscale, yscale;     // multiplier factors: 1 and s2, or 1/T and s2 T for FastDT codes
-    AhatArgs p[kMaxBatch];
 };
+template <int NP>
+struct AhatBatchOf : AhatHead {
+    AhatArgs p[NP];
+};
+using AhatBatch = AhatBatchOf<kMaxBatch>;
 cudaError_t launch_ahat_pair(const AhatBatch& b, cudaStream_t st);
 // Dynamic shared memory of one A_hat pass-pair block for lines of at most nmax positions.
 size_t ahat_pass_smem_bytes(int nmax);
@@ -261,11 +295,15 @@ struct WtaFinishArgs {
     uint16_t* disp;
     long long npix, thread0;
 };
-struct WtaFinishBatch {
+struct WtaFinishHead {
     int npairs;
     long long total_threads;
-    WtaFinishArgs p[kMaxBatch];
 };
+template <int NP>
+struct WtaFinishBatchOf : WtaFinishHead {
+    WtaFinishArgs p[NP];
+};
+using WtaFinishBatch = WtaFinishBatchOf<kMaxBatch>;
 cudaError_t launch_wta_finish(const WtaFinishBatch& b, cudaStream_t st);
 // The multiplier map of a pass along rows (horiz) or columns of a W x H image: for each
 // (line, position), (ain ? ain[pix] : 1, aout ? s2 / aout[pix] : s2), ain/aout [H][W].

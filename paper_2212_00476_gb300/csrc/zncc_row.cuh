@@ -261,15 +261,17 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
             }
         }
     };
-    const int nrc = (NSR + kStatsItem - 1) / kStatsItem;
-    for (int t = tid; t < nch + nrc; t += blockDim.x) {
-        if (t < nch) {
+    // (the right runs start at a whole warp, so that no warp walks both kinds one after the other)
+    const int nrc = (NSR + kStatsItem - 1) / kStatsItem, right0 = (nch + 31) & ~31;
+    for (int t = tid; t < right0 + nrc; t += blockDim.x) {
+        if (t < right0) {
+            if (t >= nch) continue;
             const uint4* const col = LP + lpos(t * kL);
             int2* const out = SL + lpos(t * kL);
             stats(std::integral_constant<int, kL>(), [&](int u) { return col[u + (u >> 4) * lpad]; },
                   [&](int i, int S, float is) { out[i] = make_int2(S, __float_as_int(is * lscale)); });
         } else {
-            const int c = (t - nch) * kStatsItem;                       // first centre, from c0
+            const int c = (t - right0) * kStatsItem;                       // first centre, from c0
             const CostArray<PAD, uint4> col = RP.from(c);               // (its first column is c0 + c - R = xr0 + c)
             const CostArray<PAD, int2> out = SR.from(c);
             stats(std::integral_constant<int, kStatsItem>(), [&](int u) { return col.at(u); },
@@ -435,7 +437,8 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
 // and visits them row by row, at most spb slices per visit, so that the band of a row is
 // staged once per visit and every block gets the same work within one unit.
 template <int R, typename T, int MODE, int MINB, bool SINGLE>
-__global__ void __launch_bounds__(MINB == 2 ? 320 : 512, MINB) k_zncc_row(const __grid_constant__ RowBatch b) {
+__global__ void __launch_bounds__(MINB == 2 ? 320 : 512, MINB) 
+k_zncc_row(const __grid_constant__ RowBatchOf<SINGLE ? 1 : kMaxBatch> b) {
     extern __shared__ uint4 smem_u4[];
     __shared__ unsigned long long bar;                  // bulk copies of the image rows (HPair)
     unsigned phase = 0;
@@ -508,20 +511,21 @@ inline bool zncc_row_bulk_fits(int R, const RowArgs& a) {
 }
 
 template <int R, int MINB, bool SINGLE>
-static void (*row_fn_t(int mode, int dtype))(RowBatch) {
+static const void* row_fn_t(int mode, int dtype) {
     if (mode == kModeRaw)
-        return dtype == 0 ? k_zncc_row<R, float, kModeRaw, MINB, SINGLE> : k_zncc_row<R, __half, kModeRaw, MINB, SINGLE>;
+        return dtype == 0 ? (const void*)k_zncc_row<R, float, kModeRaw, MINB, SINGLE>
+                          : (const void*)k_zncc_row<R, __half, kModeRaw, MINB, SINGLE>;
     if (mode == kModeHPair)
-        return dtype == 0 ? k_zncc_row<R, float, kModeHPair, MINB, SINGLE>
-                          : dtype == 1 ? k_zncc_row<R, __half, kModeHPair, MINB, SINGLE>
-                                       : k_zncc_row<R, uint8_t, kModeHPair, MINB, SINGLE>;
-    return k_zncc_row<R, float, kModeWta, MINB, SINGLE>;
+        return dtype == 0   ? (const void*)k_zncc_row<R, float, kModeHPair, MINB, SINGLE>
+               : dtype == 1 ? (const void*)k_zncc_row<R, __half, kModeHPair, MINB, SINGLE>
+                            : (const void*)k_zncc_row<R, uint8_t, kModeHPair, MINB, SINGLE>;
+    return (const void*)k_zncc_row<R, float, kModeWta, MINB, SINGLE>;
 }
 
 // Batched launches come from the fused path only (HPair, Wta); a batched Raw launch would
 // use the single-pair variant's arguments and is never made.
 template <int R>
-static void (*row_fn(int mode, int dtype, bool minb2, bool single))(RowBatch) {
+static const void* row_fn(int mode, int dtype, bool minb2, bool single) {
     if (single) return minb2 ? row_fn_t<R, 2, true>(mode, dtype) : row_fn_t<R, 1, true>(mode, dtype);
     if (mode == kModeRaw) return nullptr;
     return minb2 ? row_fn_t<R, 2, false>(mode, dtype) : row_fn_t<R, 1, false>(mode, dtype);
@@ -532,9 +536,9 @@ static void (*row_fn(int mode, int dtype, bool minb2, bool single))(RowBatch) {
 template <int R>
 cudaError_t zncc_row_occupancy_impl(int mode, int dtype, int threads, size_t smem, bool minb2, bool single,
                                     int* bps) {
-    void (*fn)(RowBatch) = row_fn<R>(mode, dtype, minb2, single);
+    const void* fn = row_fn<R>(mode, dtype, minb2, single);
     if (!fn) return cudaErrorInvalidValue;
-    cudaError_t e = set_max_smem((const void*)fn, smem);
+    cudaError_t e = set_max_smem(fn, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, fn, threads, smem);
 }
@@ -542,14 +546,14 @@ cudaError_t zncc_row_occupancy_impl(int mode, int dtype, int threads, size_t sme
 template <int R>
 cudaError_t launch_zncc_row_impl(const RowBatch& b, int threads, size_t smem, int mode, int dtype,
                                  cudaStream_t st) {
-    void (*fn)(RowBatch) = row_fn<R>(mode, dtype, b.p[0].minb2 != 0, b.npairs == 1);
+    const void* fn = row_fn<R>(mode, dtype, b.p[0].minb2 != 0, b.npairs == 1);
     if (!fn) return cudaErrorInvalidValue;
-    cudaError_t e = set_max_smem((const void*)fn, smem);
+    cudaError_t e = set_max_smem(fn, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config(cfg, attr, dim3(b.grid), dim3(threads), smem, st, 1);
-    return cudaLaunchKernelEx(&cfg, fn, b);
+    return b.npairs == 1 ? launch_batch(cfg, fn, first_pair<RowHead>(b)) : launch_batch(cfg, fn, b);
 }
 
 }  // namespace zncc
