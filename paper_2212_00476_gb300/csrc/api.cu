@@ -708,7 +708,10 @@ void add_line_pair(LineBatch& b, const LineArgs& ai, int mode, int dtype, int& t
 //    90 us a pass with 4 lanes, 66 with 8).
 //  - lines per block: columns in fours for 64-byte pixels, so that a row of the box is 256
 //    bytes of DRAM (1280x384x128 F32, columns per block: 4 88.9 us, 2 89.7, 1 104), rows one
-//    by one (a row's slab is contiguous anyway). Blocks of more than 512 threads get 96
+//    by one (a row's slab is contiguous anyway).
+//  - two columns to a warp (F32, scan groups of four chunks): V pair + WTA 64 -> 58 us, columns of
+//    192 pixels 20 -> 16 us a pass.
+//  - threads: blocks of more than 512 threads get 96
 //    registers a thread instead of 128; a store pass in F32 loses more by that than two columns
 //    gain (columns of 1080: one column per block 752 us, two in 576 threads 797), the WTA pass
 //    and half storage gain (WTA there: 653 and 504 us).
@@ -717,18 +720,19 @@ void add_line_pair(LineBatch& b, const LineArgs& ai, int mode, int dtype, int& t
 bool dt_lines_shape(const zncc_ctx* c, const LinePass& p, int scan, DtShape& best) {
     const int n = p.horiz ? c->W : c->H, elem = p.dtype == 0 ? 4 : 2;
     const int most = p.mode == kLineWta || p.dtype == 1 ? kDtThreads : 512;
+    const int lpc = p.v_lpc > 0 && !p.horiz && p.mode == kLineStore ? p.v_lpc : 8;
     for (int lanes = 8; lanes >= 2; lanes /= 2) {
-        const int nch = padded_chunks(n, lanes), per_line = nch * lanes;
-        if (scan * lanes > 32 || per_line > most || kG * lanes > (1 << p.sd_shift)) continue;
-        int lines = p.horiz ? 1 : 256 / (kG * lanes * elem);
-        if (p.v_lpc > 0 && !p.horiz && p.mode == kLineStore) lines = std::min(lines, p.v_lpc);
-        for (; lines >= 1; --lines) {
-            if (lines * per_line > most) continue;
-            for (int nco = 2; nco >= 1; --nco) {
-                DtShape s{lanes, scan, lines, nch, nco, p.horiz ? 1 : 0};
-                if (dt_lines_layout(p.dtype, p.mulmap != nullptr, s) > (size_t)c->smem_max) continue;
-                best = s;
-                return true;
+        if (scan * lanes > 32 || kG * lanes > (1 << p.sd_shift)) continue;
+        for (int cols = !p.horiz && p.dtype == 0 && lanes == 4 && scan == 4 && lpc > 1 ? 2 : 1; cols >= 1; --cols) {
+            const int nch = padded_chunks(n, lanes * cols), per_line = nch * lanes * cols;
+            for (int lines = p.horiz ? 1 : std::min(lpc, 256 / (kG * lanes * elem)); lines >= cols; lines -= cols) {
+                if (lines / cols * per_line > most) continue;
+                for (int nco = 2; nco >= 1; --nco) {
+                    DtShape s{lanes, scan, lines, cols, nch, nco, p.horiz ? 1 : 0};
+                    if (dt_lines_layout(p.dtype, p.mulmap != nullptr, s) > (size_t)c->smem_max) continue;
+                    best = s;
+                    return true;
+                }
             }
         }
     }
@@ -780,7 +784,7 @@ zncc_status run_dt_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* pa
         b.drill = lc->wait_drill;
         for (int i = first; i < n; ++i) {
             const DtShape& t = shapes[i];
-            if (done[i] || t.lanes != s.lanes || t.scan != s.scan || t.lines != s.lines || t.nch != s.nch ||
+            if (done[i] || t.lanes != s.lanes || t.scan != s.scan || t.lines != s.lines || t.cols != s.cols || t.nch != s.nch ||
                 t.nco != s.nco || (i != first && (alone || fills_device(ctxs[i]))))
                 continue;
             done[i] = true;
@@ -810,12 +814,12 @@ zncc_status run_dt_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* pa
             b.total_steps += a.ngroups * a.nsl;
         }
         const size_t smem = dt_lines_layout(dtype, passes[first].mulmap != nullptr, b.s);
-        const int threads = s.lines * s.nch * s.lanes;
+        const int threads = s.lines / s.cols * b.s.per_line;
         int bps = 0;
-        ZNCC_CUDA(lc, cached_occupancy(lc, 4, (((long long)mode * 4 + dtype) * 16 + s.lanes) * 2 + (b.npairs == 1), (long long)smem * 1024 + threads,
+        ZNCC_CUDA(lc, cached_occupancy(lc, 4, ((((long long)mode * 4 + dtype) * 16 + s.lanes) * 2 + s.cols - 1) * 2 + (b.npairs == 1), (long long)smem * 1024 + threads,
                                        [&](int* v) {
                                            return (dtype == 0 ? dt_lines_occupancy_f32 : dt_lines_occupancy_f16)(
-                                               mode, s.lanes, threads, smem, b.npairs == 1, v);
+                                               mode, s, threads, smem, b.npairs == 1, v);
                                        },
                                        &bps), "occupancy query");
         b.grid = std::max(1, std::min(b.total_steps, lc->num_sms * std::max(1, bps)));

@@ -79,15 +79,21 @@ struct StepWta {
     }
 };
 
-template <typename T, int MODE, int lanes, int NP, int MAXT>
+// COLS = 2: the lanes of a chunk in shuffles are those of two adjacent columns (lane bits: dq,
+// column, chunk), so that a quarter warp reads 128 contiguous bytes of a box of 64-byte pixels
+// (with eight chunks of one column per warp two chunks share each bank group) and chunks pad
+// to four per line instead of eight. "Line" below then stands for the pair of columns that share a
+// barrier and scan buffers.
+template <typename T, int MODE, int lanes, int COLS, int NP, int MAXT>
 __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBatch<NP> b) {
     constexpr bool SINGLE = NP == 1;
-    constexpr int ds = kG * lanes, cpw = 32 / lanes;     // disparities per step, chunks per warp
+    constexpr int ds = kG * lanes;                       // disparities per step
+    constexpr int LC = lanes * COLS, cpw = 32 / LC;      // lanes per chunk in shuffles, chunks per warp
     extern __shared__ __align__(128) unsigned char dt_smem[];
     __shared__ unsigned long long full[kDtThreads / 32], empty[kDtThreads / 32], drill_bar;
     if (threadIdx.x < b.s.nwl) {            // per warp of a line: its chunks' boxes, their readers
         mbar_init(&full[threadIdx.x], (unsigned)cpw);
-        mbar_init(&empty[threadIdx.x], (unsigned)b.s.lines);
+        mbar_init(&empty[threadIdx.x], (unsigned)(b.s.lines / COLS));
     }
     // (tests) the wait drill, as in k_line_pair
     if (b.drill && threadIdx.x == 0) mbar_init(&drill_bar, 1);
@@ -133,24 +139,27 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
     Cursor o = rest;
     if (SINGLE && full_rounds > 0) o = Cursor{0, (int)blockIdx.x, 0};
 
-    // this thread's place: line li of the group, warp w of the line, chunk k, lane dq of the chunk
+    // this thread's place: line li of the group (column col of the pair), warp w of the line, chunk k,
+    // lane dq of the chunk
     const int li = threadIdx.x / b.s.per_line;
     const int w = (threadIdx.x - li * b.s.per_line) >> 5;
     const int lane = threadIdx.x & 31;
-    const int dq = lane & (lanes - 1), k = w * cpw + lane / lanes;
+    const int dq = lane & (lanes - 1), k = w * cpw + lane / LC;
+    const int col = COLS > 1 ? lane / lanes & (COLS - 1) : 0, lc = li * COLS + col;      // column of the group
     // shared memory: [staging][coefficients: nco per line][multipliers: nco][scan buffers]
     unsigned char* const base = dt_smem + (-smem_addr(dt_smem) & 127u);      // (a tensor copy's alignment)
-    const T* const mine = reinterpret_cast<T*>(base) + k * b.s.slot + li * b.s.line_off + dq * kG;
-    float4* const co_mine = reinterpret_cast<float4*>(base + b.s.co_off) + li * b.s.nco * b.s.arr;     // this line's
-    float2* const mul_mine = reinterpret_cast<float2*>(base + b.s.mul_off) + li * b.s.nco * b.s.arr;
-    float4* const sb = reinterpret_cast<float4*>(base + b.s.scan_off) + li * 2 * b.s.nvg * lanes + dq;
+    const T* const mine = reinterpret_cast<T*>(base) + k * b.s.slot + lc * b.s.line_off + dq * kG;
+    float4* const co_mine = reinterpret_cast<float4*>(base + b.s.co_off) + lc * b.s.nco * b.s.arr;     // this column's
+    float2* const mul_mine = reinterpret_cast<float2*>(base + b.s.mul_off) + lc * b.s.nco * b.s.arr;
+    float4* const sb = reinterpret_cast<float4*>(base + b.s.scan_off) + li * 2 * b.s.nvg * LC + (lane & (LC - 1));
     float* const sa = reinterpret_cast<float*>(base + b.s.scan_off + b.s.lines * 2 * b.s.nvg * lanes * 16) +
-                      li * 2 * b.s.nvg * lanes + dq;
+                      li * 2 * b.s.nvg * LC + (lane & (LC - 1));
 
     auto prefetch_coef = [&](const Cursor& q, int cbuf) {
         const DtArgs& a = P(q.pi);
-        const int ln = q.g * b.s.lines + li;
-        for (int t = w * 32 + lane; t < b.s.nch * kL; t += b.s.per_line) {
+        const int ln = q.g * b.s.lines + lc;
+        // (each column's own lanes copy its coefficients)
+        for (int t = COLS > 1 ? k * lanes + dq : w * 32 + lane; t < b.s.nch * kL; t += b.s.per_line / COLS) {
             const bool in = ln < a.nlines && t < a.n;
             const size_t at = (size_t)ln * a.n + t;
             cp_async<16>(co_mine + cbuf * b.s.arr + cpos(t), in ? a.coef + at : a.coef, in);
@@ -171,7 +180,7 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
         const int at = k * kL, line0 = q.g * b.s.lines;
         tma_load_4d(dst, m, dd, b.s.horiz ? at : line0, b.s.horiz ? line0 : at, slab, bar);
     };
-    if (li == 0 && dq == 0 && left > 0) load_box(o);
+    if (lc == 0 && dq == 0 && left > 0) load_box(o);
     if (b.s.nco == 2) prefetch_coef(o, 0);
 
     StepWta<lanes> wr;
@@ -210,13 +219,13 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
 #pragma unroll
             for (int i = 0; i < kL; ++i) mul4<true>(mul[i].x, v[i]);
         }
-        dt_group_pair<MODE != kLineWta, true, lanes>(v, co, lanes, b.s.scan_shift, lane, k, b.s.nvg, sa, sb, b.s2, mul, 1 + li, b.s.per_line,
+        dt_group_pair<MODE != kLineWta, true, LC>(v, co, LC, b.s.scan_shift, lane, k, b.s.nvg, sa, sb, b.s2, mul, 1 + li, b.s.per_line,
             [&]() {
                 // the box has been read: the lines' warps say so, and its loader refills it
                 __syncwarp();
-                if (b.s.lines > 1 && lane == 0) mbar_arrive(&empty[w]);
-                if (li == 0 && dq == 0 && left > 1) {
-                    if (b.s.lines > 1 && !mbar_wait(&empty[w], par, kBulkWaitPolls)) {
+                if (b.s.lines > COLS && lane == 0) mbar_arrive(&empty[w]);
+                if (lc == 0 && dq == 0 && left > 1) {
+                    if (b.s.lines > COLS && !mbar_wait(&empty[w], par, kBulkWaitPolls)) {
                         atomicOr(b.fault, kFaultTmaWait);
                         mbar_wait(&empty[w], par, kBulkWaitPolls);
                     }
@@ -227,7 +236,7 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
             });
         const int dl = o.sl * ds + dq * kG;
         const int nvalid = max(0, min(4, a.dcount - dl));
-        const int line = o.g * b.s.lines + li;
+        const int line = o.g * b.s.lines + lc;
         if constexpr (MODE == kLineWta) {
             wr.fold(v, nvalid, dl, dq);
             if (o.sl == a.nsl - 1 || left == 1) {
@@ -261,7 +270,7 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
 size_t dt_lines_layout(int dtype, bool mul, DtShape& s) {
     const int elem = dtype == 0 ? 4 : 2, ds = kG * s.lanes;
     s.mul = mul;
-    s.per_line = s.nch * s.lanes;
+    s.per_line = s.nch * s.lanes * s.cols;
     s.nwl = s.per_line / 32;
     s.nvg = s.nch / s.scan;
     s.scan_shift = 0;
@@ -273,7 +282,7 @@ size_t dt_lines_layout(int dtype, bool mul, DtShape& s) {
     s.co_off = s.nch * s.slot * elem;
     s.mul_off = s.co_off + s.lines * s.nco * s.arr * 16;
     s.scan_off = s.mul_off + (mul ? s.lines * s.nco * s.arr * 8 : 0);
-    return 128 + (size_t)s.scan_off + (size_t)s.lines * 2 * s.nvg * s.lanes * 20;
+    return 128 + (size_t)s.scan_off + (size_t)s.lines * 2 * s.nvg * s.lanes * 20;   // (lines / cols sets of lanes * cols)
 }
 #define DT_NAME(f) f##_f32
 using DtElem = float;
@@ -282,37 +291,38 @@ using DtElem = float;
 using DtElem = __half;
 #endif
 
-template <int NP, int MAXT>
-static void (*dt_lines_fn_t(int mode, int lanes))(DtBatch<NP>) {
-    if (mode == kLineStore)
-        return lanes == 8   ? k_dt_lines<DtElem, kLineStore, 8, NP, MAXT>
-               : lanes == 4 ? k_dt_lines<DtElem, kLineStore, 4, NP, MAXT>
-                            : k_dt_lines<DtElem, kLineStore, 2, NP, MAXT>;
-    return lanes == 8   ? k_dt_lines<DtElem, kLineWta, 8, NP, MAXT>
-           : lanes == 4 ? k_dt_lines<DtElem, kLineWta, 4, NP, MAXT>
-                        : k_dt_lines<DtElem, kLineWta, 2, NP, MAXT>;
+template <int MODE, int NP, int MAXT>
+static const void* dt_lines_fn_t(int lanes, int cols) {
+    if constexpr (std::is_same<DtElem, float>::value)
+        if (cols == 2) return lanes == 4 ? (const void*)k_dt_lines<DtElem, MODE, 4, 2, NP, MAXT> : nullptr;
+    return lanes == 8   ? (const void*)k_dt_lines<DtElem, MODE, 8, 1, NP, MAXT>
+           : lanes == 4 ? (const void*)k_dt_lines<DtElem, MODE, 4, 1, NP, MAXT>
+                        : (const void*)k_dt_lines<DtElem, MODE, 2, 1, NP, MAXT>;
 }
 template <int NP>
-static void (*dt_lines_fn(int mode, int lanes, int threads))(DtBatch<NP>) {
-    return threads <= 512 ? dt_lines_fn_t<NP, 512>(mode, lanes) : dt_lines_fn_t<NP, kDtThreads>(mode, lanes);
+static const void* dt_lines_fn(int mode, int lanes, int cols, int threads) {
+    if (mode == kLineStore)
+        return threads <= 512 ? dt_lines_fn_t<kLineStore, NP, 512>(lanes, cols) : dt_lines_fn_t<kLineStore, NP, kDtThreads>(lanes, cols);
+    return threads <= 512 ? dt_lines_fn_t<kLineWta, NP, 512>(lanes, cols) : dt_lines_fn_t<kLineWta, NP, kDtThreads>(lanes, cols);
 }
 
-cudaError_t DT_NAME(dt_lines_occupancy)(int mode, int lanes, int threads, size_t smem, bool single, int* blocks_per_sm) {
-    const void* fn = single ? (const void*)dt_lines_fn<1>(mode, lanes, threads)
-                            : (const void*)dt_lines_fn<kMaxBatch>(mode, lanes, threads);
+cudaError_t DT_NAME(dt_lines_occupancy)(int mode, const DtShape& s, int threads, size_t smem, bool single,
+                                        int* blocks_per_sm) {
+    const void* fn = single ? dt_lines_fn<1>(mode, s.lanes, s.cols, threads)
+                            : dt_lines_fn<kMaxBatch>(mode, s.lanes, s.cols, threads);
     cudaError_t e = set_max_smem(fn, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
 }
 
 cudaError_t DT_NAME(launch_dt_lines)(const DtBatch<kMaxBatch>& b, size_t smem, int mode, cudaStream_t st) {
-    const int threads = b.s.lines * b.s.nch * b.s.lanes;
+    const int threads = b.s.lines / b.s.cols * b.s.per_line;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     launch_config(cfg, attr, dim3(b.grid), dim3(threads), smem, st, 1);
     const bool single = b.npairs == 1;
-    const void* fn = single ? (const void*)dt_lines_fn<1>(mode, b.s.lanes, threads)
-                            : (const void*)dt_lines_fn<kMaxBatch>(mode, b.s.lanes, threads);
+    const void* fn = single ? dt_lines_fn<1>(mode, b.s.lanes, b.s.cols, threads)
+                            : dt_lines_fn<kMaxBatch>(mode, b.s.lanes, b.s.cols, threads);
     cudaError_t e = set_max_smem(fn, smem);
     if (e != cudaSuccess) return e;
     if (!single) return launch_batch(cfg, fn, b);

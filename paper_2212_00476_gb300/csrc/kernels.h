@@ -155,11 +155,12 @@ struct DtArgs {
 struct DtShape {
     int lanes;                // lanes per chunk (4 disparities each): a slice is 4 * lanes disparities
     int scan;                 // chunks per scan group: the carries' association (a power of two)
-    int lines;                // adjacent lines per block
+    int lines;                // adjacent lines per block, a multiple of cols
+    int cols;                 // adjacent lines that share warps (1 or 2)
     int nch;                  // chunks per line, padded to whole warps
     int nco;                  // coefficient buffers per line (1 or 2)
     int horiz;
-    // filled by dt_lines_layout: multipliers in use, threads and warps per line, scan groups per
+    // filled by dt_lines_layout: multipliers in use, threads and warps per cols lines, scan groups per
     // line, entries of a chunk's box, between its positions and between its lines, of a line's
     // coefficient array, and byte offsets in shared memory
     int scan_shift, mul, per_line, nwl, nvg, slot, ps, line_off, arr, co_off, mul_off, scan_off;
@@ -178,8 +179,8 @@ struct DtBatch : DtHead {
 // Completes a shape; returns the dynamic shared memory of its blocks.
 size_t dt_lines_layout(int dtype, bool mul, DtShape& s);
 constexpr int kDtThreads = 640;               // the most threads of a block
-cudaError_t dt_lines_occupancy_f32(int mode, int lanes, int threads, size_t smem, bool single, int* blocks_per_sm);
-cudaError_t dt_lines_occupancy_f16(int mode, int lanes, int threads, size_t smem, bool single, int* blocks_per_sm);
+cudaError_t dt_lines_occupancy_f32(int mode, const DtShape& s, int threads, size_t smem, bool single, int* blocks_per_sm);
+cudaError_t dt_lines_occupancy_f16(int mode, const DtShape& s, int threads, size_t smem, bool single, int* blocks_per_sm);
 cudaError_t launch_dt_lines_f32(const DtBatch<kMaxBatch>& b, size_t smem, int mode, cudaStream_t st);
 cudaError_t launch_dt_lines_f16(const DtBatch<kMaxBatch>& b, size_t smem, int mode, cudaStream_t st);
 
