@@ -343,16 +343,10 @@ zncc_status run_coef(zncc_ctx* lc, const PairIO* io, int n, float sigma_s, float
 // Lanes per 16-pixel chunk in the cost kernel: the warps of a row in 512 threads.
 int row_lanes(int W) { return W <= 1024 ? 8 : (W <= 2048 ? 4 : 2); }
 
-// Whether a context's cost kernel takes the two-blocks-per-SM variant (blocks of at most 320
-// threads): the second block hides the first one's latencies and barriers, but both stage the
-// rows that they visit, so it takes two units (row, slice) per block (us of the cost kernel with
-// one and two blocks: 640x192, D = 64, 1.3 units 29 and 31; 1242x375, D = 32, 2.5 units 49 and
-// 46; 1280x384, D = 128, 10 units 120 and 106; 600x1000, D = 40, 6.6 units 91 and 64). Not with
-// WTA alone, whose rows are whole units and whose running best spills there.
-bool row_two_blocks(const zncc_ctx* c, int mode) {
-    if (c->row_minb2) return c->row_minb2 == 1;
-    const int tq = row_lanes(c->W), nslices = (c->D + kG * tq - 1) / (kG * tq);
-    return mode != kModeWta && (long long)c->H * nslices >= 4ll * c->num_sms;
+// Units (row, disparity slice) of a pair in the cost kernel.
+long long row_units(const zncc_ctx* c) {
+    const int ds = kG * row_lanes(c->W);
+    return (long long)c->H * ((c->D + ds - 1) / ds);
 }
 
 // Cost-kernel launches over the pairs (one per window radius among them). A block covers
@@ -376,13 +370,27 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
         b.fault = lc->fault;
         int threads = 0;
         size_t smem = 0;
-        // two blocks per SM where every pair of the launch allows it
-        bool minb2 = nch0 * tq0 <= 320;
-        for (int i = first; i < n; ++i) minb2 = minb2 && (done[i] || row_two_blocks(io[i].c, mode));
+        auto shares = [&](int i) {
+            return !done[i] && io[i].c->r == r && row_lanes(io[i].c->W) == tq0 && padded_chunks(io[i].c->W, tq0) == nch0 &&
+                   (i == first || !(alone || fills_device(io[i].c)));
+        };
+        // Two blocks per SM (of at most 320 threads): the second block hides the first one's
+        // latencies and barriers, but both stage the rows that they visit, so it takes two units
+        // per block (us of the cost kernel with one and two blocks: 640x192, D = 64, 1.3 units 29
+        // and 31; 1242x375, D = 32, 2.5 units 49 and 46; 1280x384, D = 128, 10 units 120 and 106;
+        // 600x1000, D = 40, 6.6 units 91 and 64). Not with WTA alone, whose rows are whole units
+        // and whose running best spills there.
+        long long units = 0;
+        bool all_two = true, any_one = false;
+        for (int i = first; i < n; ++i)
+            if (shares(i)) {
+                units += row_units(io[i].c);
+                all_two = all_two && io[i].c->row_minb2 == 1;
+                any_one = any_one || io[i].c->row_minb2 == 2;
+            }
+        const bool minb2 = nch0 * tq0 <= 320 && (all_two || (!any_one && mode != kModeWta && units >= 4ll * lc->num_sms));
         for (int i = first; i < n; ++i) {
-            if (done[i] || io[i].c->r != r || row_lanes(io[i].c->W) != tq0 || padded_chunks(io[i].c->W, tq0) != nch0 ||
-                (i != first && (alone || fills_device(io[i].c))))
-                continue;
+            if (!shares(i)) continue;
             done[i] = true;
             zncc_ctx* c = io[i].c;
             RowArgs& a = b.p[b.npairs++];
