@@ -75,3 +75,28 @@ def test_slab_passes_in_a_batch(storage):
         c.set_tuning(Z.ZNCC_TUNE_LINE_LOADS, 1)
         assert torch.equal(o, run(c, l, r, 2, storage))
         c.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("w,h,d,off", [(1, 1, 8, 0), (40, 384, 16, 0), (41, 385, 24, 0), (375, 130, 40, 0), (1280, 20, 32, 0),
+                                       (1281, 9, 64, 0), (200, 193, 128, 0), (200, 193, 100, 0), (64, 50, 20, 0),
+                                       (64, 50, 17, 0), (64, 50, 32, 1), (64, 50, 32, 4), (7, 450, 8, 0)])
+def test_aggregation_of_a_callers_volume_equals_general_passes(w, h, d, off, storage):
+    """dt_aggregate with and without the TMA-staged passes (by pixel alignment, start address and
+    line length): the same sums in the same association, so the same values bit for bit."""
+    rng = np.random.default_rng(w + h + d + off)
+    tdt = torch.float32 if storage == "f32" else torch.float16
+    guide = dev(rng.integers(0, 256, (h, w), dtype=np.uint8) // 16 * 3)
+    v = torch.from_numpy(rng.uniform(-1, 1, (h, w, d)).astype(np.float32)).cuda()
+    with Z.ZnccContext(w, h, d, 3) as ctx:
+        got = []
+        for loads in (0, 1):
+            buf = torch.zeros(off + h * w * d, dtype=tdt, device="cuda")
+            cost = buf[off:].view(h, w, d)
+            cost.copy_(v)
+            ctx.set_tuning(Z.ZNCC_TUNE_LINE_LOADS, loads)
+            ctx.dt_aggregate(guide, cost, 20.0, 0.3, 2, STORAGE[storage])
+            torch.cuda.synchronize()
+            got.append(cost.clone())
+        assert ctx.device_faults() == 0
+    assert torch.equal(got[0], got[1])
