@@ -832,6 +832,11 @@ zncc_status run_dt_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* pa
                                        },
                                        &bps), "occupancy query");
         b.grid = std::max(1, std::min(b.total_steps, lc->num_sms * std::max(1, bps)));
+        // One chunk's lanes carry through the scan groups of long F32 rows (14 warps and more, W >
+        // 1664) that a block has many steps of (us a pass without and with it: 1920x1080x256, 106
+        // steps, 709 and 636; 1920x1080x64, 28 steps, 182 and 175; 1800x400x128, 21 steps, 123 and
+        // 130; 1600x1080x256, 13 warps, 546 and 572); columns lose by it.
+        b.s.chain = s.horiz && b.s.nwl >= 14 && b.total_steps >= 24 * b.grid;
         ZNCC_LAUNCH(lc, kind, (dtype == 0 ? launch_dt_lines_f32 : launch_dt_lines_f16)(b, smem, mode, lc->cur), "DT pass pair");
     }
     return ZNCC_OK;

@@ -588,9 +588,13 @@ __device__ __forceinline__ void dt_pair(float (&v)[kL][4], const float4* __restr
 // (LANES where known at compile time, else lanes). k: this thread's chunk of the line; sa / sb:
 // the line's scan buffers, 2 * nvg * lanes entries each, at this thread's lane of the chunk; bar:
 // the barrier of the line's bar_threads threads (0 with the whole block: the block's).
-template <bool SCALE, bool PACKED, int LANES, typename Hook, typename MulT>
+// CHAIN and chain: the lanes of the first chunk carry through all of the groups once and leave
+// every group's carry in shared memory (nvg * lanes float4 after sb's), instead of every thread
+// walking the groups before its own: one more barrier a phase for a walk that the warps of a long
+// line otherwise make many times over.
+template <bool SCALE, bool PACKED, int LANES, bool CHAIN = false, typename Hook, typename MulT>
 __device__ __forceinline__ void dt_group_pair(float (&v)[kL][4], const float4* __restrict__ co, int lanes_, int scan_shift, int lane,
-                                              int k, int nvg, float* sa, float4* sb, float s2,
+                                              int k, int nvg, bool chain, float* sa, float4* sb, float s2,
                                               const MulT* __restrict__ mul, int bar, int bar_threads,
                                               Hook after_read) {
     const int lanes = LANES ? LANES : lanes_;
@@ -639,11 +643,28 @@ __device__ __forceinline__ void dt_group_pair(float (&v)[kL][4], const float4* _
     named_barrier(bar, bar_threads);
 
     // ---- phase 2: carry from the groups before, corrected forward values, backward sweep ----
+    if (CHAIN && chain) {
+        if (k == 0) {
+            float4* const out = sb + 2 * nvg * lanes;
+#pragma unroll 4
+            for (int g = 0; g < nvg; ++g) {
+                const float4 b2 = sb[g * lanes];
+                const float a2 = sa[g * lanes];
+                out[g * lanes] = make_float4(F[0], F[1], F[2], F[3]);
+                const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
+                fma4<PACKED>(a2, F, b4, F);
+            }
+        }
+        named_barrier(bar, bar_threads);
+        const float4 f = sb[(2 * nvg + vg) * lanes];
+        F[0] = f.x; F[1] = f.y; F[2] = f.z; F[3] = f.w;
+    } else {
 #pragma unroll 1
-    for (int g = 0; g < vg; ++g) {
-        const float4 b2 = sb[g * lanes];
-        const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
-        fma4<PACKED>(sa[g * lanes], F, b4, F);
+        for (int g = 0; g < vg; ++g) {
+            const float4 b2 = sb[g * lanes];
+            const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
+            fma4<PACKED>(sa[g * lanes], F, b4, F);
+        }
     }
     fma4<PACKED>(Ae, F, Be, F);
     float h[4] = {0.f, 0.f, 0.f, 0.f};
@@ -688,11 +709,28 @@ __device__ __forceinline__ void dt_group_pair(float (&v)[kL][4], const float4* _
     named_barrier(bar, bar_threads);
 
     // ---- phase 3: carry from the groups after, backward correction, scale ----
+    if (CHAIN && chain) {
+        if (k == 0) {
+            float4* const out = sb + 2 * nvg * lanes;
+#pragma unroll 4
+            for (int g = nvg - 1; g >= 0; --g) {
+                const float4 b2 = sb2[g * lanes];
+                const float a2 = sa2[g * lanes];
+                out[g * lanes] = make_float4(G[0], G[1], G[2], G[3]);
+                const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
+                fma4<PACKED>(a2, G, b4, G);
+            }
+        }
+        named_barrier(bar, bar_threads);
+        const float4 f = sb[(2 * nvg + vg) * lanes];
+        G[0] = f.x; G[1] = f.y; G[2] = f.z; G[3] = f.w;
+    } else {
 #pragma unroll 1
-    for (int g = nvg - 1; g > vg; --g) {
-        const float4 b2 = sb2[g * lanes];
-        const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
-        fma4<PACKED>(sa2[g * lanes], G, b4, G);
+        for (int g = nvg - 1; g > vg; --g) {
+            const float4 b2 = sb2[g * lanes];
+            const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
+            fma4<PACKED>(sa2[g * lanes], G, b4, G);
+        }
     }
     fma4<PACKED>(Ae, G, Be, G);
     if (SCALE && (mul || s2 != 1.0f)) {

@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
     constexpr bool SINGLE = NP == 1;
     constexpr int ds = kG * lanes;                       // disparities per step
     constexpr int LC = lanes * COLS, cpw = 32 / LC;      // lanes per chunk in shuffles, chunks per warp
+    constexpr bool kChain = MODE == kLineStore && MAXT <= 512;      // (the 96-register variants would spill)
     extern __shared__ __align__(128) unsigned char dt_smem[];
     __shared__ unsigned long long full[kDtThreads / 32], empty[kDtThreads / 32], drill_bar;
     if (threadIdx.x < b.s.nwl) {            // per warp of a line: its chunks' boxes, their readers
@@ -151,8 +152,8 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
     const T* const mine = reinterpret_cast<T*>(base) + k * b.s.slot + lc * b.s.line_off + dq * kG;
     float4* const co_mine = reinterpret_cast<float4*>(base + b.s.co_off) + lc * b.s.nco * b.s.arr;     // this column's
     float2* const mul_mine = reinterpret_cast<float2*>(base + b.s.mul_off) + lc * b.s.nco * b.s.arr;
-    float4* const sb = reinterpret_cast<float4*>(base + b.s.scan_off) + li * 2 * b.s.nvg * LC + (lane & (LC - 1));
-    float* const sa = reinterpret_cast<float*>(base + b.s.scan_off + b.s.lines * 2 * b.s.nvg * lanes * 16) +
+    float4* const sb = reinterpret_cast<float4*>(base + b.s.scan_off) + li * 3 * b.s.nvg * LC + (lane & (LC - 1));
+    float* const sa = reinterpret_cast<float*>(base + b.s.scan_off + b.s.lines * 3 * b.s.nvg * lanes * 16) +
                       li * 2 * b.s.nvg * LC + (lane & (LC - 1));
 
     auto prefetch_coef = [&](const Cursor& q, int cbuf) {
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
 #pragma unroll
             for (int i = 0; i < kL; ++i) mul4<true>(mul[i].x, v[i]);
         }
-        dt_group_pair<MODE != kLineWta, true, LC>(v, co, LC, b.s.scan_shift, lane, k, b.s.nvg, sa, sb, b.s2, mul, 1 + li, b.s.per_line,
+        dt_group_pair<MODE != kLineWta, true, LC, kChain>(v, co, LC, b.s.scan_shift, lane, k, b.s.nvg, b.s.chain != 0, sa, sb, b.s2, mul, 1 + li, b.s.per_line,
             [&]() {
                 // the box has been read: the lines' warps say so, and its loader refills it
                 __syncwarp();
@@ -270,6 +271,7 @@ __global__ void __launch_bounds__(MAXT) k_dt_lines(const __grid_constant__ DtBat
 size_t dt_lines_layout(int dtype, bool mul, DtShape& s) {
     const int elem = dtype == 0 ? 4 : 2, ds = kG * s.lanes;
     s.mul = mul;
+    s.chain = 0;
     s.per_line = s.nch * s.lanes * s.cols;
     s.nwl = s.per_line / 32;
     s.nvg = s.nch / s.scan;
@@ -282,7 +284,7 @@ size_t dt_lines_layout(int dtype, bool mul, DtShape& s) {
     s.co_off = s.nch * s.slot * elem;
     s.mul_off = s.co_off + s.lines * s.nco * s.arr * 16;
     s.scan_off = s.mul_off + (mul ? s.lines * s.nco * s.arr * 8 : 0);
-    return 128 + (size_t)s.scan_off + (size_t)s.lines * 2 * s.nvg * s.lanes * 20;   // (lines / cols sets of lanes * cols)
+    return 128 + (size_t)s.scan_off + (size_t)s.lines * s.nvg * s.lanes * (3 * 16 + 2 * 4);   // (lines / cols sets of lanes * cols)
 }
 #define DT_NAME(f) f##_f32
 using DtElem = float;

@@ -163,6 +163,7 @@ struct DtShape {
     // filled by dt_lines_layout: multipliers in use, threads and warps per cols lines, scan groups per
     // line, entries of a chunk's box, between its positions and between its lines, of a line's
     // coefficient array, and byte offsets in shared memory
+    int chain;                // one chunk's lanes carry through the scan groups (dt_group_pair; by the launcher)
     int scan_shift, mul, per_line, nwl, nvg, slot, ps, line_off, arr, co_off, mul_off, scan_off;
 };
 struct DtHead {

@@ -366,7 +366,7 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
             float4* const sb = reinterpret_cast<float4*>(sm + a.sb_off);
             float* const sa = reinterpret_cast<float*>(sm + a.sa_off);
             const int shift = 5 - a.tq_shift, nvg = nthr >> 5;      // scan groups: the warps
-            dt_group_pair<kFast, PAD, 0>(v, co + k * kCS, tq, shift, t3 & 31, k, nvg, sa + dq, sb + dq, kFast ? a.s2 : 1.0f,
+            dt_group_pair<kFast, PAD, 0>(v, co + k * kCS, tq, shift, t3 & 31, k, nvg, false, sa + dq, sb + dq, kFast ? a.s2 : 1.0f,
                                           kFast ? mrow + k * kCS : (const float*)nullptr, 0, nthr, NoHook());
         }
         const int x0 = k * kL, d_first = a.d_lo + sl * ds + dq * kG;

@@ -100,3 +100,16 @@ def test_aggregation_of_a_callers_volume_equals_general_passes(w, h, d, off, sto
             got.append(cost.clone())
         assert ctx.device_faults() == 0
     assert torch.equal(got[0], got[1])
+
+
+def test_carries_through_long_rows_with_many_steps():
+    """Rows of 14 warps and more with many steps per block: one chunk's lanes carry through the scan
+    groups."""
+    w, h, d = 1700, 80, 800
+    p = make_pair(h, w, d, seed=11, disp="planes")
+    left, right = dev(p.left), dev(p.right)
+    with Z.ZnccContext(w, h, d, 3) as ctx:
+        new = run(ctx, left, right, 2, "f32")
+        ctx.set_tuning(Z.ZNCC_TUNE_LINE_LOADS, 1)
+        ref = run(ctx, left, right, 2, "f32")
+    assert torch.equal(new, ref)
