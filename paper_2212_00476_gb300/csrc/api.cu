@@ -36,11 +36,12 @@ void set_free_error(const char* fmt, ...) {
 }  // namespace
 
 // Every device allocation of the library goes through here. Host-side fault injection for
-// tests: with the environment variable ZNCC_FAIL_DEVICE_ALLOC set to 1, each allocation
-// reports cudaErrorMemoryAllocation without calling the driver (no GPU fault is involved).
+// tests: with the environment variable ZNCC_FAIL_DEVICE_ALLOC set to 1, each allocation, and set
+// to ">N", each one of more than N bytes, reports cudaErrorMemoryAllocation without calling the
+// driver (no GPU fault is involved).
 cudaError_t zncc::device_alloc(void** p, size_t bytes) {
     const char* f = getenv("ZNCC_FAIL_DEVICE_ALLOC");
-    if (f && f[0] == '1') {
+    if (f && (f[0] == '1' || (f[0] == '>' && bytes > strtoull(f + 1, nullptr, 10)))) {
         *p = nullptr;
         return cudaErrorMemoryAllocation;
     }
@@ -93,6 +94,7 @@ struct zncc_ctx {
     unsigned long long* keys = nullptr;   // [H][W] fused-WTA keys, zero between runs
     void* vol = nullptr;          // the fused path's intermediate volume (on first use)
     size_t vol_bytes = 0;
+    bool compact = false;         // the volume's pixels are padded to 4 entries, not to whole slabs
     float* ahat = nullptr;        // [nahat][H][W] DT responses of an all-ones plane (F16, I8 storage)
     float2* mulmap = nullptr;     // [nmul] maps of the pairs from 2 (F16) or 1 (I8) on:
     int nahat = 0, nmul = 0;      //        (A_hat_{p-1}, s2 / A_hat_p), line-major
@@ -859,7 +861,7 @@ int slab_shift(int dtype) { return dtype == 0 ? 4 : 5; }
 const float2 kSomeMul{};          // stands for a multiplier map where only its presence counts
 
 bool slab_path(zncc_ctx* c, int dtype, bool norm) {
-    if (c->line_loads != 0 || dtype == 2 || !tmap_encoder()) return false;
+    if (c->line_loads != 0 || dtype == 2 || c->compact || !tmap_encoder()) return false;
     for (int k = 0; k < 3; ++k) {                   // rows, columns, columns with WTA
         LinePass p;
         p.dcount = c->D;
@@ -946,13 +948,29 @@ zncc_status run_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* passe
     return ZNCC_OK;
 }
 
-zncc_status ensure_volume(zncc_ctx* c, int dtype, long long dstride) {
-    const size_t need = (size_t)c->W * c->H * (size_t)dstride * (dtype == 0 ? 4 : (dtype == 1 ? 2 : 1));
+zncc_status ensure_volume_bytes(zncc_ctx* c, size_t need) {
     if (c->vol_bytes >= need) return ZNCC_OK;
     free_dev(c->vol);
     c->vol_bytes = 0;
     ZNCC_TRY(alloc_dev(c, &c->vol, need, "cost volume"));
     c->vol_bytes = need;
+    return ZNCC_OK;
+}
+
+// The volume of a fused run: whole slabs, whatever the plan in use (a captured run keeps its
+// buffer when the plan changes). Where the device has no memory for them, the context keeps the
+// compact volume (and k_line_pair's passes) from now on.
+zncc_status ensure_volume(zncc_ctx* c, int dtype) {
+    const size_t npix = (size_t)c->W * c->H;
+    if (!c->compact) {
+        const zncc_status st = ensure_volume_bytes(c, npix * slab_pixel_bytes(c->D, dtype));
+        if (st != ZNCC_ENOMEM || dtype == 2) return st;
+    }
+    ZNCC_TRY(ensure_volume_bytes(c, npix * compact_pixel_bytes(c->D, dtype)));
+    if (dtype != 2 && !c->compact) {
+        c->compact = true;
+        c->err.clear();
+    }
     return ZNCC_OK;
 }
 
@@ -1126,18 +1144,15 @@ zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigm
     const int dt = storage;                         // 0 float, 1 half, 2 FastDT codes
     zncc_ctx* ctxs[kMaxBatch];
     bool slabs = true;
-    for (int i = 0; i < n; ++i) slabs = slabs && slab_path(io[i].c, dt, dt == 1 && iters > 1);
     for (int i = 0; i < n; ++i) {
         ctxs[i] = io[i].c;
-        io[i].dstride = (io[i].c->D + 3) / 4 * 4;     // padded so that every access is vectorised
-        long long entries = io[i].dstride;
-        if (slabs) {
-            io[i].sd_shift = slab_shift(dt);
-            io[i].dstride = 1 << io[i].sd_shift;
-            entries = (io[i].c->D + io[i].dstride - 1) / io[i].dstride * io[i].dstride;
-        }
-        if (ensure_volume(io[i].c, dt, entries) != ZNCC_OK) return fail(lc, ZNCC_ENOMEM, io[i].c->err);
+        if (ensure_volume(io[i].c, dt) != ZNCC_OK) return fail(lc, ZNCC_ENOMEM, io[i].c->err);
         io[i].vol = io[i].c->vol;
+        slabs = slabs && slab_path(io[i].c, dt, dt == 1 && iters > 1);
+    }
+    for (int i = 0; i < n; ++i) {
+        if (slabs) io[i].sd_shift = slab_shift(dt);
+        io[i].dstride = slabs ? 1 << io[i].sd_shift : compact_entries(io[i].c->D);
     }
     const float K = (float)exp(-1.0 / (double)sigma_s);
     const float inv_sr255 = (float)(1.0 / (255.0 * (double)sigma_r));
@@ -1271,6 +1286,12 @@ zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigm
     ZNCC_LAUNCH(lc, K_WTA_FINISH, launch_wta_finish(fb, lc->cur), "WTA finish");
     return ZNCC_OK;
 }
+
+}  // namespace
+
+void zncc::keep_compact_volume(zncc_ctx* c) { c->compact = true; }
+
+namespace {
 
 // ---- dt_aggregate_noalloc: per-device state of the static scratch --------------------
 // Everything here has static storage: the device limits, read once per device, and a

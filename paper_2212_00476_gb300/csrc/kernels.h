@@ -405,8 +405,22 @@ cudaError_t launch_plane(const PlaneBatch& b, int cls, size_t smem, cudaStream_t
 cudaError_t launch_fastdt_codec(const int16_t* values, int n, uint8_t* codes, int16_t* decoded, cudaStream_t st);
 
 // Device allocation of the library (cudaMalloc, or an injected out-of-memory failure when the
-// environment variable ZNCC_FAIL_DEVICE_ALLOC is 1).
+// environment variable ZNCC_FAIL_DEVICE_ALLOC asks for one).
 cudaError_t device_alloc(void** p, size_t bytes);
+
+// Bytes of the volume per pixel in a fused run's context: whole slabs of 64 bytes (F32, F16), or
+// padded to four entries (I8, and contexts that keep the compact volume, whose line passes are
+// k_line_pair's).
+inline size_t volume_entry_bytes(int dtype) { return dtype == 0 ? 4 : (dtype == 1 ? 2 : 1); }
+inline int compact_entries(int D) { return (D + 3) / 4 * 4; }     // every access is vectorised
+inline size_t compact_pixel_bytes(int D, int dtype) { return compact_entries(D) * volume_entry_bytes(dtype); }
+inline size_t slab_pixel_bytes(int D, int dtype) {
+    return dtype == 2 ? compact_pixel_bytes(D, dtype) : (D * volume_entry_bytes(dtype) + 63) / 64 * 64;
+}
+}  // namespace zncc
+struct zncc_ctx;
+namespace zncc {
+void keep_compact_volume(zncc_ctx* c);
 
 // Scratch of dt_aggregate_noalloc: the DT coefficients of one W x H image (two float4 per
 // pixel) in a static device array of this size; its address on the current device.

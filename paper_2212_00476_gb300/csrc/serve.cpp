@@ -51,13 +51,13 @@ struct ShapeKey {
 };
 
 // Device bytes a context of this shape holds: DT coefficients (two float4 per pixel), the
-// fused WTA's keys, the volume (pixel stride padded to 4 entries), the A_hat maps and
-// multipliers of the F16 and I8 paths, the images and map.
-size_t shape_charge(const ShapeKey& k) {
+// fused WTA's keys, the volume (whole slabs, or compact: pixels padded to 4 entries), the A_hat maps
+// and multipliers of the F16 and I8 paths, the images and map.
+size_t shape_charge(const ShapeKey& k, bool compact) {
     const size_t npix = (size_t)k.W * k.H;
     size_t b = 32 * npix + 8 * npix + 4 * npix;
     if (k.iters > 0) {
-        b += npix * (size_t)((k.D + 3) / 4 * 4) * (k.storage == ZNCC_F32 ? 4 : (k.storage == ZNCC_F16 ? 2 : 1));
+        b += npix * (compact ? zncc::compact_pixel_bytes(k.D, k.storage) : zncc::slab_pixel_bytes(k.D, k.storage));
         if (k.storage == ZNCC_F16 && k.iters > 1) b += npix * 12 * (size_t)(2 * k.iters - 1);
         if (k.storage == ZNCC_I8) b += npix * (4 * (size_t)(2 * k.iters - 1) + 8 * (size_t)(2 * k.iters));
     }
@@ -207,7 +207,7 @@ bool reserve(zncc_server* s, size_t need, std::vector<Slot*>& victims) {
 // A new context and its buffers for this shape, or nullptr with *st set. Makes CUDA calls
 // that may synchronize the device: never under the lock (a batch's completion function
 // needs the lock, so waiting for the device while holding it would never end).
-Slot* create_slot(const ShapeKey& key, size_t charge, zncc_status* st, char* err, size_t errlen) {
+Slot* create_slot(const ShapeKey& key, size_t charge, bool compact, zncc_status* st, char* err, size_t errlen) {
     Slot* sl = new Slot();
     sl->key = key;
     sl->charge = charge;
@@ -216,6 +216,7 @@ Slot* create_slot(const ShapeKey& key, size_t charge, zncc_status* st, char* err
     if (*st != ZNCC_OK) {
         snprintf(err, errlen, "context for a request: %s", zncc_last_error(nullptr));
     } else {
+        if (compact) zncc::keep_compact_volume(sl->ctx);
         cudaError_t e = zncc::device_alloc((void**)&sl->d_img, 2 * npix);
         if (e == cudaSuccess) e = zncc::device_alloc((void**)&sl->d_disp, npix * sizeof(uint16_t));
         if (e != cudaSuccess) {
@@ -390,7 +391,9 @@ void worker_main(zncc_server* s) {
             Slot* sl = take_idle(s, r->key);
             if (!sl) {
                 std::vector<Slot*> victims;
-                const size_t need = shape_charge(r->key);
+                // a shape whose slabs alone exceed the budget keeps the compact volume
+                const bool compact = shape_charge(r->key, false) > s->budget;
+                const size_t need = shape_charge(r->key, compact);
                 if (!reserve(s, need, victims)) break;          // wait for room, in order
                 s->queue.erase(s->queue.begin() + (long)idx);
                 r->state = Request::RUNNING;
@@ -398,7 +401,7 @@ void worker_main(zncc_server* s) {
                 for (Slot* v : victims) destroy_slot(v);
                 zncc_status st = ZNCC_OK;
                 char err[256];
-                sl = create_slot(r->key, need, &st, err, sizeof(err));
+                sl = create_slot(r->key, need, compact, &st, err, sizeof(err));
                 lk.lock();
                 if (!sl) {                                      // cannot run: fail it, go on
                     s->charged -= need;
@@ -493,10 +496,10 @@ zncc_status serve_submit(zncc_server* s, const uint8_t* left_host, const uint8_t
         return st;
     }
     ShapeKey key{width, height, max_disp, win, (int)storage, iters};
-    if (shape_charge(key) > s->budget) {                        // could never be admitted
+    if (shape_charge(key, true) > s->budget) {                        // could never be admitted
         std::lock_guard<std::mutex> lk(s->mu);
         snprintf(s->err, sizeof(s->err), "serve_submit: the request needs %zu bytes of device memory, "
-                 "more than the budget of %zu", shape_charge(key), s->budget);
+                 "more than the budget of %zu", shape_charge(key, true), s->budget);
         return ZNCC_EINVAL;
     }
     const size_t npix = (size_t)width * height;
