@@ -189,7 +189,9 @@ zncc_status fastdt_codec(const int16_t* values, int n, uint8_t* codes, int16_t* 
  * volume is written once per horizontal/vertical hand-over and never read back for WTA.
  * iters == 0 computes ZNCC and WTA in one kernel without storing any volume.
  * `storage` is the type of the context-owned intermediate volume (F16 halves its traffic,
- * I8 quarters it at some loss of accuracy: the FastDT storage above).
+ * I8 quarters it at some loss of accuracy: the FastDT storage above). Its pixels are padded to
+ * whole multiples of 64 bytes (F32, F16) where the device has memory for that, to four entries
+ * otherwise; the map does not depend on it.
  * left/right: device images; disp: device uint16 [H][W]. Sec. V-C fuses ZNCC with L2R and
  * WTA with D2U in the same way. */
 zncc_status zncc_run(zncc_ctx* ctx, const uint8_t* left, const uint8_t* right, int pitch,
@@ -240,7 +242,8 @@ zncc_status zncc_run_host(zncc_ctx* ctx, const uint8_t* left_host, const uint8_t
  * Results are identical to running each pair alone: the batched kernels compute every pair
  * exactly as a single zncc_run does. Contexts are reused per request shape; the device memory
  * they hold (cost volume, DT coefficients, A_hat maps, images and disparity map) is charged
- * to `volume_budget_bytes`, and idle ones are freed, least recently used first, when a new
+ * to `volume_budget_bytes` (a shape that fits only without the volume's padding to 64 bytes per
+ * pixel runs without it), and idle ones are freed, least recently used first, when a new
  * shape needs room. The paper has no serving layer; the batched path serves its workload of
  * many independent pairs. All server calls are thread-safe, except that no call may run
  * concurrently with or after serve_destroy. */
@@ -327,8 +330,9 @@ const char* zncc_status_string(zncc_status status);
  *   ZNCC_TUNE_ROW_SPB    cost kernel: disparity slices per block
  *   ZNCC_TUNE_H_TQ       horizontal DT pairs: lanes per 16-pixel chunk (2, 4 or 8)
  *   ZNCC_TUNE_V_TQ       vertical DT pairs: lanes per 16-pixel chunk (2, 4 or 8)
- *   ZNCC_TUNE_AHAT_SMS   (F16, I8 storage) SMs the cost kernel leaves free for the A_hat chain,
- *                        which runs beside it on a second stream (default 8)
+ *   ZNCC_TUNE_AHAT_SMS   (F16, I8 storage, ZNCC_TUNE_ROW_MINB2 = 1) SMs the cost kernel leaves
+ *                        free for the A_hat chain, which runs beside it on a second stream
+ *                        (default 8)
  *   ZNCC_TUNE_PLANE      (F32 storage, iters >= 1) 1 = the plane-resident path for pairs with
  *                        W <= 1024 whose rows split into bands of at most 32 rows over a
  *                        cluster of 1, 2, 4 or 8 CTAs that fit in shared memory (H <= 256):

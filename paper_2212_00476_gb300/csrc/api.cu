@@ -1164,8 +1164,7 @@ zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigm
     const bool literal = dt == 0 && 4.0 * iters * -log(1.0 - (double)K) <= log(1e30);
     const float s2 = literal ? 1.0f : scale_s2(sigma_s);
     // The DT weights of the line pairs (and the A_hat maps) depend only on the guide; they are
-    // computed first, on the same stream: the persistent cost kernel fills every SM, so work
-    // on a second stream would only run after it anyway. The cost kernel computes the
+    // computed beside the cost kernel on a second stream. The cost kernel computes the
     // coefficients of its own rows and stores them for the later horizontal pairs, so the
     // coefficient kernel computes the columns' only.
     // Half storage keeps each stored pair p >= 2 divided by A_hat_p (the per-pixel bound of
@@ -1188,11 +1187,11 @@ zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigm
     // and costs where it does not (1920x1080x256: 5.73 -> 6.10 ms, the passes waiting for
     // free SMs), so it is taken where the pass needs at most 64 KB of shared memory, or as
     // ZNCC_TUNE_AHAT_JOIN says. FastDT's pairs measured slower that way (1.21 -> 1.23 ms), so
-    // there pair 2 waits for the whole side stream, as without multipliers. The cost kernel's
-    // 128-register variant holds one block per SM and leaves registers and shared memory for
-    // the side kernels' blocks on every SM; its two-blocks-per-SM variant fills the registers,
-    // so with the A_hat chain `reserve` SMs are left to it. FastDT needs A_hat_1 in the cost
-    // kernel itself, so that pass comes first, on the main stream.
+    // there pair 2 waits for the whole side stream, as without multipliers. (Both measured with
+    // k_line_pair's passes.) Where two cost blocks per SM are asked for (ZNCC_TUNE_ROW_MINB2 = 1),
+    // `reserve` SMs are left to the A_hat chain; where the kernel takes them by itself nothing is
+    // reserved, since the run is level either way (1242x375x128 F16: 420 us with 0 and with 8).
+    // FastDT needs A_hat_1 in the cost kernel itself, so that pass comes first, on the main stream.
     const int reserve = norm && lc->row_minb2 == 1 ? (lc->ahat_sms > 0 ? lc->ahat_sms : kAhatSideSms) : 0;
     int p_first_side = 1;
     if (dt == 2) {

@@ -20,9 +20,9 @@ namespace zncc {
 //
 // Bound by HBM for F32 store passes: a pass moves the volume once in and once out, and an
 // in-place pass of a plain kernel over the same bytes takes 78-82 us at 1280x384x128. Measured
-// there (k_line_pair -> this kernel, us): columns 94 -> 89, rows 95 -> 85, last columns with WTA
-// 75 -> 63; F16 at 1242x375x128: columns 77 -> 60, rows 110 -> 64, WTA 84 -> 53; F32 at
-// 1920x1080x256: columns 1188 -> 731, rows 888 -> 710, WTA 790 -> 506.
+// there (k_line_pair -> this kernel, us): columns 94 -> 87, rows 95 -> 86, last columns with WTA
+// 75 -> 58; F16 at 1242x375x128: columns 77 -> 60, rows 110 -> 64, WTA 84 -> 53; F32 at
+// 1920x1080x256: columns 1188 -> 735, rows 888 -> 636, WTA 790 -> 510.
 //
 // Staging: one lane per chunk copies the box of the next step's chunk (all lines of the group)
 // into shared memory by TMA as soon as the lines' warps have read the last one into registers,
