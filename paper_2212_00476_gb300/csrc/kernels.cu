@@ -191,8 +191,59 @@ k_window_stats(const uint8_t* __restrict__ img, int pitch, int W, int H, int x_b
     }
 }
 
+// The statistics of a small image, one block per row: every pixel of a column's window is read
+// for each of its rows, but nothing is carried from row to row, so that the chain of dependent
+// steps is a fraction of k_window_stats's. Bound by launch and latency.
+__global__ void k_window_stats_row(const uint8_t* __restrict__ img, int pitch, int W, int H, int r,
+                                   int x_begin, int nx, int* __restrict__ S, int* __restrict__ Q,
+                                   float* __restrict__ isig, int2* __restrict__ packed) {
+    extern __shared__ int sm_stats[];
+    const int y = blockIdx.x;
+    const int ncol = nx + 2 * r;
+    int* cs = sm_stats;
+    int* cq = sm_stats + ncol;
+    for (int t = threadIdx.x; t < ncol; t += blockDim.x) {
+        const int xc = min(max(x_begin - r + t, 0), W - 1);
+        int s = 0, q = 0;
+        for (int j = -r; j <= r; ++j) {
+            const int p = img[(size_t)min(max(y + j, 0), H - 1) * pitch + xc];
+            s += p;
+            q += p * p;
+        }
+        cs[t] = s;
+        cq[t] = q;
+    }
+    __syncthreads();
+    const unsigned n = (unsigned)((2 * r + 1) * (2 * r + 1));
+    for (int t = threadIdx.x; t < nx; t += blockDim.x) {
+        int s = 0, q = 0;
+        for (int i = 0; i <= 2 * r; ++i) {
+            s += cs[t + i];
+            q += cq[t + i];
+        }
+        const size_t o = (size_t)y * nx + t;
+        const int var = (int)(n * (unsigned)q - (unsigned)s * (unsigned)s);
+        const float is = var > 0 ? rsqrtf((float)var) : 0.0f;
+        if (S) S[o] = s;
+        if (Q) Q[o] = q;
+        if (isig) isig[o] = is;
+        if (packed) packed[o] = make_int2(s, __float_as_int(is));
+    }
+}
+
+// Below this many pixel reads (centres x rows of the window) the row kernel is faster (us, row
+// kernel and k_window_stats, back to back: 206x179 9x9, 0.3 M reads, 4.6 and 8.3; 514x687 9x9,
+// 3.2 M, 6.5 and 10.7; 653x482 13x13, 4.1 M, 8.3 and 10.5; 816x981 7x7, 5.6 M, 10.5 and 8.4;
+// 752x733 13x13, 7.2 M, 10.4 and 8.5; 1840x754 11x11, 15 M, 16.7 and 10.5).
+constexpr long long kStatsRowReads = 5000000;
+
 cudaError_t launch_window_stats(const uint8_t* img, int pitch, int W, int H, int r, int x_begin,
                                 int nx, int* S, int* Q, float* isig, int2* packed, cudaStream_t st) {
+    if ((long long)nx * H * (2 * r + 1) < kStatsRowReads) {
+        const size_t smem = 2 * sizeof(int) * (size_t)(nx + 2 * r);
+        k_window_stats_row<<<H, 256, smem, st>>>(img, pitch, W, H, r, x_begin, nx, S, Q, isig, packed);
+        return cudaGetLastError();
+    }
     const dim3 grid((nx + stats_centres(r) - 1) / stats_centres(r), (H + kStatsRows - 1) / kStatsRows);
     // four pixels a load where the rows start on 4 bytes; four results a store where every
     // output row starts on 16

@@ -39,6 +39,14 @@ def test_window_stats_tiles_and_alignment(w, h, r, off, pad):
     assert np.allclose(inv.cpu().numpy(), ref, rtol=4e-7, atol=0)
 
 
+# the same where the image is large enough for the kernel that walks down the rows (5 M pixel reads)
+@pytest.mark.parametrize("w,h,r,off,pad", [
+    (1667, 1000, 1, 0, 1), (1666, 1000, 1, 4, 2), (1012, 1009, 2, 0, 0), (499, 1121, 5, 2, 1), (500, 1024, 5, 0, 4),
+    (494, 777, 7, 0, 2), (495, 775, 7, 1, 1), (1920, 1080, 5, 0, 0), (1001, 556, 4, 3, 7)])
+def test_window_stats_of_large_images(w, h, r, off, pad):
+    test_window_stats_tiles_and_alignment(w, h, r, off, pad)
+
+
 # D around the lanes per pixel and loads per lane, volumes that start off 16 bytes
 @pytest.mark.parametrize("dtype", ["f32", "f16"])
 @pytest.mark.parametrize("d,off", [(1, 0), (2, 0), (3, 1), (8, 0), (8, 1), (31, 0), (32, 0), (33, 0), (36, 2),
