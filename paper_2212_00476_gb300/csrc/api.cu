@@ -411,8 +411,6 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
             a.dstride = io[i].dstride;
             a.sd_shift = io[i].sd_shift;
             a.slab_stride = (long long)c->W * c->H * io[i].dstride;
-            a.vec = io[i].vol && (io[i].dstride % 4 == 0) &&
-                    ((uintptr_t)io[i].vol % (dtype == 0 ? 16 : (dtype == 1 ? 8 : 4)) == 0) ? 1 : 0;
             a.mulmap = io[i].mulmap1;
             a.K = K;
             a.inv_sr255 = inv_sr255;
@@ -1450,7 +1448,9 @@ zncc_status zncc_cost_volume(zncc_ctx* c, const uint8_t* left, const uint8_t* ri
     if (!cost) return fail(c, ZNCC_EINVAL, "cost pointer is NULL");
     if (dtype != ZNCC_F32 && dtype != ZNCC_F16) return fail(c, ZNCC_EINVAL, "unknown dtype");
     PairIO io{c, left, right, pitch, nullptr, cost, c->D};
-    return run_rows(c, &io, 1, kModeRaw, dtype, 0.0f, 0.0f, 0.0f, K_ZNCC_RAW, 0, "ZNCC cost");
+    // groups of four entries go out together where every pixel's groups are aligned
+    const bool groups = c->D % 4 == 0 && (uintptr_t)cost % (dtype == ZNCC_F32 ? 16 : 8) == 0;
+    return run_rows(c, &io, 1, groups ? kModeRaw : kModeRawAny, dtype, 0.0f, 0.0f, 0.0f, K_ZNCC_RAW, 0, "ZNCC cost");
 }
 
 }  // extern "C"

@@ -127,6 +127,9 @@ __device__ __forceinline__ void st4(__half* p, int nvalid, bool vec, const float
     }
 }
 
+__device__ __forceinline__ void st1(float* p, float o) { *p = o; }
+__device__ __forceinline__ void st1(__half* p, float o) { *p = __float2half_rn(o); }
+
 // ---- FastDT storage (Sec. IV-C): 8-bit codes of near-zero-mean 16-bit costs -------------
 // A stored value is E = rint(kFastT * (v(d_arb) - v(d)) / A_hat) as a 16-bit integer
 // (values that do no better than d_arb, E >= 0, are 0); its code keeps the six bits next to

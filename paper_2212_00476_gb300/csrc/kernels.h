@@ -7,7 +7,9 @@
 
 namespace zncc {
 
-enum { kModeRaw = 0, kModeHPair = 1, kModeWta = 2 };   // k_zncc_row variants
+// k_zncc_row variants: the costs alone (Raw: pixels aligned to whole groups of four entries; RawAny: any
+// volume), with the row's DT pass pair, or with WTA
+enum { kModeRaw = 0, kModeHPair = 1, kModeWta = 2, kModeRawAny = 3 };
 enum { kLineStore = 0, kLineWta = 1 };                  // k_line_pair variants
 constexpr int kMaxBatch = 32;                           // pairs per batched launch
 
@@ -31,7 +33,6 @@ struct RowArgs {
     long long dstride;        // entries per pixel in the output
     int sd_shift;             // disparity d is entry d mod 2^sd_shift of slab d >> sd_shift ...
     long long slab_stride;    // ... and a slab is this many entries
-    int vec;                  // 16-byte (float) / 8-byte (half) accesses allowed
     float K, inv_sr255;       // DT weights (HPair): exp(-1/sigma_s), 1/(255 sigma_r); guide = left
     float4* coefH_out;        // (HPair) if set, the row coefficients go here too ([H][W], as k_dt_coef)
     const float2* mulmap;     // (HPair, FastDT codes) [H][W]: (unused, output scale (1-K)^2/A_hat_1)

@@ -280,7 +280,6 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
     }
     __syncthreads();
 
-    const bool vec = a.vec != 0;
     WtaRegs wr;
     if constexpr (MODE == kModeWta) wr.reset();
 
@@ -393,14 +392,48 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
                     q += a.dstride;
                 }
             }
+        } else if constexpr (MODE == kModeRawAny) {
+            // Pixels off the alignment of whole groups are stored one entry at a time. Four lanes (the
+            // two of a chunk with tq = 2) first trade their 4 x 4 (2 x 4) entries, so that a store
+            // instruction writes four (two) adjacent entries of each chunk instead of every fourth one
+            // and a 32-byte sector is written in fewer pieces (us a call, every fourth entry and this:
+            // 1280x384x127 F32 276 and 186, 1296x315x246 F16 414 and 258, 2500x700x61 F32 672 and 568).
+            // (A block is whole warps, all of them here.)
+            const bool quad = tq >= 4;
+            const int l = dq & (quad ? 3 : 1);
+            const int left = a.d_hi - (d_first - 3 * l);     // entries from the first that this lane stores
+            T* p = q - 3 * l;
+            const int o2 = quad ? 8 : 2, o3 = o2 + 4;
+#pragma unroll
+            for (int i = 0; i < kL; ++i) {
+                float e[4] = {v[i][0], v[i][1], v[i][2], v[i][3]};
+                const float r0 = __shfl_xor_sync(kFull, l & 1 ? e[0] : e[1], 1);
+                const float r1 = __shfl_xor_sync(kFull, l & 1 ? e[2] : e[3], 1);
+                if (l & 1) { e[0] = r0; e[2] = r1; } else { e[1] = r0; e[3] = r1; }
+                if (quad) {
+                    const float r2 = __shfl_xor_sync(kFull, l & 2 ? e[0] : e[2], 2);
+                    const float r3 = __shfl_xor_sync(kFull, l & 2 ? e[1] : e[3], 2);
+                    if (l & 2) { e[0] = r2; e[1] = r3; } else { e[2] = r2; e[3] = r3; }
+                }
+                if (x0 + i < W) {
+                    if (0 < left) st1(p, e[0]);
+                    if (4 < left) st1(p + 4, e[1]);
+                    if (o2 < left) st1(p + o2, e[2]);
+                    if (o3 < left) st1(p + o3, e[3]);
+                }
+                p += a.dstride;
+            }
         } else if (nvalid > 0) {
-            if (vec && nvalid == 4 && x0 + kL <= W) {        // a whole chunk of whole groups
+            // (Raw: the costs are finished before the first store; interleaved, the addresses would
+            // not fit in 96 registers beside the tile)
+            if constexpr (MODE == kModeRaw && PAD) asm volatile("" ::: "memory");
+            if (nvalid == 4 && x0 + kL <= W) {               // a whole chunk of whole groups
 #pragma unroll
                 for (int i = 0; i < kL; ++i) st4(q + (size_t)i * a.dstride, 4, true, v[i]);
             } else {
 #pragma unroll
                 for (int i = 0; i < kL; ++i) {
-                    if (x0 + i < W) st4(q, nvalid, vec, v[i]);
+                    if (x0 + i < W) st4(q, nvalid, true, v[i]);
                     q += a.dstride;
                 }
             }
@@ -512,9 +545,14 @@ inline bool zncc_row_bulk_fits(int R, const RowArgs& a) {
 
 template <int R, int MINB, bool SINGLE>
 static const void* row_fn_t(int mode, int dtype) {
-    if (mode == kModeRaw)
-        return dtype == 0 ? (const void*)k_zncc_row<R, float, kModeRaw, MINB, SINGLE>
-                          : (const void*)k_zncc_row<R, __half, kModeRaw, MINB, SINGLE>;
+    if constexpr (SINGLE) {
+        if (mode == kModeRaw)
+            return dtype == 0 ? (const void*)k_zncc_row<R, float, kModeRaw, MINB, true>
+                              : (const void*)k_zncc_row<R, __half, kModeRaw, MINB, true>;
+        if (mode == kModeRawAny)
+            return dtype == 0 ? (const void*)k_zncc_row<R, float, kModeRawAny, MINB, true>
+                              : (const void*)k_zncc_row<R, __half, kModeRawAny, MINB, true>;
+    }
     if (mode == kModeHPair)
         return dtype == 0   ? (const void*)k_zncc_row<R, float, kModeHPair, MINB, SINGLE>
                : dtype == 1 ? (const void*)k_zncc_row<R, __half, kModeHPair, MINB, SINGLE>
@@ -527,7 +565,7 @@ static const void* row_fn_t(int mode, int dtype) {
 template <int R>
 static const void* row_fn(int mode, int dtype, bool minb2, bool single) {
     if (single) return minb2 ? row_fn_t<R, 2, true>(mode, dtype) : row_fn_t<R, 1, true>(mode, dtype);
-    if (mode == kModeRaw) return nullptr;
+    if (mode == kModeRaw || mode == kModeRawAny) return nullptr;
     return minb2 ? row_fn_t<R, 2, false>(mode, dtype) : row_fn_t<R, 1, false>(mode, dtype);
 }
 
