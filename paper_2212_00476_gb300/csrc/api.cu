@@ -112,7 +112,7 @@ struct zncc_ctx {
     int plane_force_cs = 0;       // its cluster size (0 = automatic)
     int plane_cs = -1;            // chosen cluster size (0: streaming path; -1: not chosen yet)
     int plane_cls = 0, plane_smem = 0, plane_clusters = 0;   // its size class, shared memory, clusters
-    int num_sms = 0;
+    int num_sms = 0, l2_bytes = 0;
     std::vector<LinePlan> plans;  // line-pass launch shapes, by pass signature
     std::vector<OccEntry> occ;    // occupancy answers
     // encoded tensor maps of the DT pairs' inputs, by (volume, pixel stride, element size,
@@ -366,93 +366,124 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
         const int r = io[first].c->r;
         const int tq0 = row_lanes(io[first].c->W), nch0 = padded_chunks(io[first].c->W, tq0);
         const bool alone = fills_device(io[first].c);
-        RowBatch b;
-        static_cast<RowHead&>(b) = RowHead{};
-        b.mode = mode;
-        b.fault = lc->fault;
-        int threads = 0;
-        size_t smem = 0;
-        auto shares = [&](int i) {
-            return !done[i] && io[i].c->r == r && row_lanes(io[i].c->W) == tq0 && padded_chunks(io[i].c->W, tq0) == nch0 &&
-                   (i == first || !(alone || fills_device(io[i].c)));
-        };
-        // Two blocks per SM (of at most 320 threads): the second block hides the first one's
-        // latencies and barriers, but both stage the rows that they visit, so it takes two units
-        // per block (us of the cost kernel with one and two blocks: 640x192, D = 64, 1.3 units 29
-        // and 31; 1242x375, D = 32, 2.5 units 49 and 46; 1280x384, D = 128, 10 units 120 and 106;
-        // 600x1000, D = 40, 6.6 units 91 and 64). Not with WTA alone, whose rows are whole units
-        // and whose running best spills there.
+        int group[kMaxBatch], members = 0;
         long long units = 0;
         bool all_two = true, any_one = false;
-        for (int i = first; i < n; ++i)
-            if (shares(i)) {
-                units += row_units(io[i].c);
-                all_two = all_two && io[i].c->row_minb2 == 1;
-                any_one = any_one || io[i].c->row_minb2 == 2;
-            }
-        const bool minb2 = nch0 * tq0 <= 320 && (all_two || (!any_one && mode != kModeWta && units >= 4ll * lc->num_sms));
         for (int i = first; i < n; ++i) {
-            if (!shares(i)) continue;
+            const zncc_ctx* c = io[i].c;
+            if (done[i] || c->r != r || row_lanes(c->W) != tq0 || padded_chunks(c->W, tq0) != nch0 ||
+                (i != first && (alone || fills_device(c))))
+                continue;
             done[i] = true;
-            zncc_ctx* c = io[i].c;
-            RowArgs& a = b.p[b.npairs++];
-            a = RowArgs{};
-            a.left = io[i].left;
-            a.right = io[i].right;
-            a.pitch = io[i].pitch;
-            a.W = c->W;
-            a.H = c->H;
-            a.D = c->D;
-            a.tq = tq0;
-            a.nch = nch0;
-            a.d_lo = 0;
-            a.d_hi = c->D;
-            a.vol = io[i].vol;
-            a.dstride = io[i].dstride;
-            a.sd_shift = io[i].sd_shift;
-            a.slab_stride = (long long)c->W * c->H * io[i].dstride;
-            a.mulmap = io[i].mulmap1;
-            a.K = K;
-            a.inv_sr255 = inv_sr255;
-            a.coefH_out = mode == kModeHPair ? c->coefH : nullptr;
-            a.s2 = s2;
-            a.minb2 = minb2 ? 1 : 0;
-            a.wta.disp = io[i].disp;
-            a.wta.first = 1;
-            a.wta.last = 1;
-            const int nthr = a.nch * a.tq;
-            const int nslices = (c->D + kG * a.tq - 1) / (kG * a.tq);
-            // WTA keeps a row's running best in registers: a block then visits whole rows. FastDT codes
-            // need slice 0 of the row in every visit, so a visit takes all the slices it can.
-            const bool whole_rows = mode == kModeWta;
-            if (whole_rows || dtype == 2) a.spb = nslices;
-            else a.spb = c->row_spb > 0 ? std::min(c->row_spb, nslices) : nslices;
-            // the image rows by bulk copies where both images and the pitch are 16-byte aligned
-            // and W is a multiple of 16, while the rows fit in the region they share and the
-            // guide row's buffer fits in shared memory; else plain loads
-            a.bulk = mode == kModeHPair && a.W % 16 == 0 && a.pitch % 16 == 0 &&
-                     (uintptr_t)a.left % 16 == 0 && (uintptr_t)a.right % 16 == 0 && !c->row_nobulk ? 1 : 0;
-            a.lpad = 1;
-            if (!minb2 && zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max) a.lpad = 0;
-            while (!whole_rows && dtype != 2 && a.spb > 1 && zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max)
-                --a.spb;
-            if (a.bulk && (zncc_row_layout(r, mode, dtype, a, nthr, minb2) > (size_t)lc->smem_max ||
-                           !zncc_row_bulk_fits_host(r, a)))
-                a.bulk = 0;
-            const size_t sm = zncc_row_layout(r, mode, dtype, a, nthr, minb2);
-            if (sm > (size_t)lc->smem_max)
-                return fail(lc, ZNCC_EUNSUPPORTED, "the cost kernel's row band does not fit in shared memory");
-            a.item0 = b.total_items;
-            a.nitems = whole_rows ? c->H : c->H * nslices;       // units: rows, or (row, slice)
-            b.total_items += a.nitems;
-            threads = std::max(threads, nthr);
-            smem = std::max(smem, sm);
+            group[members++] = i;
+            units += row_units(c);
+            all_two = all_two && c->row_minb2 == 1;
+            any_one = any_one || c->row_minb2 == 2;
         }
+        RowBatch b;
+        int threads = 0;
+        size_t smem = 0;
+        // the arguments of the group's pairs; false where a row's band does not fit in shared memory
+        auto fill = [&](bool minb2) {
+            static_cast<RowHead&>(b) = RowHead{};
+            b.mode = mode;
+            b.fault = lc->fault;
+            threads = 0;
+            smem = 0;
+            for (int m = 0; m < members; ++m) {
+                const PairIO& pio = io[group[m]];
+                zncc_ctx* c = pio.c;
+                RowArgs& a = b.p[b.npairs++];
+                a = RowArgs{};
+                a.left = pio.left;
+                a.right = pio.right;
+                a.pitch = pio.pitch;
+                a.W = c->W;
+                a.H = c->H;
+                a.D = c->D;
+                a.tq = tq0;
+                a.nch = nch0;
+                a.d_lo = 0;
+                a.d_hi = c->D;
+                a.vol = pio.vol;
+                a.dstride = pio.dstride;
+                a.sd_shift = pio.sd_shift;
+                a.slab_stride = (long long)c->W * c->H * pio.dstride;
+                a.mulmap = pio.mulmap1;
+                a.K = K;
+                a.inv_sr255 = inv_sr255;
+                a.coefH_out = mode == kModeHPair ? c->coefH : nullptr;
+                a.s2 = s2;
+                a.minb2 = minb2 ? 1 : 0;
+                a.wta.disp = pio.disp;
+                a.wta.first = 1;
+                a.wta.last = 1;
+                const int nthr = a.nch * a.tq;
+                const int nslices = (c->D + kG * a.tq - 1) / (kG * a.tq);
+                // WTA keeps a row's running best in registers: a block then visits whole rows. FastDT
+                // codes need slice 0 of the row in every visit, so a visit takes all the slices it can.
+                const bool whole_rows = mode == kModeWta;
+                if (whole_rows || dtype == 2) a.spb = nslices;
+                else a.spb = c->row_spb > 0 ? std::min(c->row_spb, nslices) : nslices;
+                // the image rows by bulk copies where both images and the pitch are 16-byte aligned
+                // and W is a multiple of 16, while the rows fit in the region they share and the
+                // guide row's buffer fits in shared memory; else plain loads
+                a.bulk = mode == kModeHPair && a.W % 16 == 0 && a.pitch % 16 == 0 &&
+                         (uintptr_t)a.left % 16 == 0 && (uintptr_t)a.right % 16 == 0 && !c->row_nobulk ? 1 : 0;
+                const size_t most = (size_t)lc->smem_max;
+                auto layout = [&]() { return zncc_row_layout(r, mode, dtype, a, nthr, minb2); };
+                a.lpad = 1;
+                if (!minb2 && layout() > most) a.lpad = 0;
+                while (!whole_rows && dtype != 2 && a.spb > 1 && layout() > most) --a.spb;
+                if (a.bulk && (layout() > most || !zncc_row_bulk_fits_host(r, a))) a.bulk = 0;
+                const size_t sm = layout();
+                if (sm > most) return false;
+                a.item0 = b.total_items;
+                a.nitems = whole_rows ? c->H : c->H * nslices;       // units: rows, or (row, slice)
+                b.total_items += a.nitems;
+                threads = std::max(threads, nthr);
+                smem = std::max(smem, sm);
+            }
+            return true;
+        };
         int bps = 0;
-        const long long k0 = ((((long long)r * 4 + mode) * 4 + dtype) * 2 + (minb2 ? 1 : 0)) * 2 + (b.npairs == 1);
-        ZNCC_CUDA(lc, cached_occupancy(lc, 1, k0 * 4096 + threads, (long long)smem, [&](int* v) {
-                      return zncc_row_occupancy(r, mode, dtype, threads, smem, minb2, b.npairs == 1, v);
-                  }, &bps), "occupancy query");
+        auto occupancy = [&](bool minb2) {
+            const long long k0 = ((((long long)r * 4 + mode) * 4 + dtype) * 2 + (minb2 ? 1 : 0)) * 2 + (b.npairs == 1);
+            return cached_occupancy(lc, 1, k0 * 4096 + threads, (long long)smem, [&](int* v) {
+                return zncc_row_occupancy(r, mode, dtype, threads, smem, minb2, b.npairs == 1, v);
+            }, &bps);
+        };
+        // Two blocks per SM (of at most 320 threads, in 96 registers): the second block hides the first
+        // one's latencies and barriers, but both stage the rows that they visit. So it takes (us of
+        // the cost kernel or volume with one and two blocks)
+        //  - two units for every resident block (640x192, D = 64, 1.3 units: 29 and 31; 320x200, D = 128,
+        //    1.3 units for four blocks of 160 threads: 13.6 and 15.0; 1242x375, D = 32, 2.5 units: 49
+        //    and 46; 1280x384, D = 128, 10 units: 120 and 106),
+        //  - shared memory for both: the variant's padded layout is the larger one, and its block alone
+        //    is slower than one of 128 registers (volume of 2304x1080, D = 64: 287 and 302),
+        //  - a volume of its own (Raw) that L2 holds, or whose pixels are whole 32-byte sectors and, in
+        //    F32, at most 20 slices: more blocks have more sectors and DRAM pages written in part,
+        //    which beyond L2 leave it like that (640x300, D = 1000 F16, 2000 bytes a pixel: 155 and
+        //    181; 1280x384, D = 124: 113 and 132; F32, D = 400, 25 slices: 178 and 184, D = 256, 16
+        //    slices: 126 and 121; in L2: 1280x720, D = 61 F16: 135 and 128).
+        // Not with WTA alone, whose rows are whole units and whose running best spills there.
+        bool two = nch0 * tq0 <= 320;
+        if (two && !all_two) {
+            const zncc_ctx* c = io[first].c;
+            const long long row = (long long)c->D * (dtype == 0 ? 4 : 2);
+            const bool scattered = mode == kModeRawAny ||
+                                   (mode == kModeRaw && (row % 32 != 0 || (dtype == 0 && c->D > 20 * kG * tq0)));
+            two = !any_one && mode != kModeWta && units >= 4ll * lc->num_sms &&
+                  !(scattered && row * c->W * c->H > lc->l2_bytes);
+        }
+        two = two && fill(true);
+        if (two && !all_two) {
+            ZNCC_CUDA(lc, occupancy(true), "occupancy query");
+            two = bps >= 2 && units >= 2ll * lc->num_sms * bps;
+        }
+        if (!two && !fill(false))
+            return fail(lc, ZNCC_EUNSUPPORTED, "the cost kernel's row band does not fit in shared memory");
+        ZNCC_CUDA(lc, occupancy(two), "occupancy query");
         b.grid = std::max(1, std::min(b.total_items, std::max(1, lc->num_sms - reserve_sms) * std::max(1, bps)));
         ZNCC_LAUNCH(lc, kind, launch_zncc_row(r, b, threads, smem, mode, dtype, lc->cur), what);
     }
@@ -1388,6 +1419,7 @@ zncc_status zncc_create(int width, int height, int max_disp, int win, zncc_ctx**
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->l2_bytes, cudaDevAttrL2CacheSize, c->device);
     const size_t npix = (size_t)width * height;
     if (e == cudaSuccess) e = device_alloc((void**)&c->coefH, npix * sizeof(float4));
     if (e == cudaSuccess) e = device_alloc((void**)&c->coefV, npix * sizeof(float4));
