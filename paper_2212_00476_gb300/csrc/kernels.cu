@@ -1036,7 +1036,7 @@ cudaError_t launch_wta_finish(const WtaFinishBatch& b, cudaStream_t st) {
 // ---------------------------------------------------------------------------------------
 // WTA over a stored volume (Sec. III-C, Eq. (WTA1)): the smallest d among the largest costs.
 // Bound by reading the volume once. LP consecutive lanes share a pixel and each reads VEC
-// entries at a time (16 bytes where the pixels are aligned), so that a warp's loads are whole
+// entries at a time (16 bytes where the pixels start on that), so that a warp's loads are whole
 // 128-byte lines and kWtaLoads of them are in flight per lane; the warp-per-pixel kernel this
 // replaces had one 4-byte load per lane in flight and five shuffle rounds per pixel
 // (1280x384x128 F32: 67.6 -> 39.2 us, 6.4 TB/s).
@@ -1076,40 +1076,120 @@ __global__ void __launch_bounds__(256) k_wta_volume(const T* __restrict__ cost, 
     if (sub == 0 && pix < npix) disp[pix] = (uint16_t)(bd == 0x7FFFFFFF ? 0 : bd);
 }
 
-// Lanes per pixel: enough that each lane has about kWtaLoads loads, so that the shuffle rounds
-// serve many entries and no load slot stays empty.
-template <typename T, int VEC>
+// The same for pixels that do not all start on 16 bytes: the aligned 16-byte vectors that a pixel's
+// entries lie in, of which the first and the last also hold entries of its neighbours (compared in
+// a branch of their own); the pixels at the ends of the volume entry by entry, so that nothing
+// around it is read. Loads of one, two or four entries took (us, and this kernel; one warp per pixel,
+// entry by entry, in brackets): 1630x458x155 F32 168 and 71 (119), F16 158 and 49 (117), 448x518x134
+// F16 50 and 13 (34), 1280x384x126 F32 43 and 41 (84), 512x400x1021 F16 112 and 80 (95).
+template <typename T, int LP>
+__global__ void __launch_bounds__(256) k_wta_volume_any(const T* __restrict__ cost, int npix, int D,
+                                                        uint16_t* __restrict__ disp) {
+    constexpr int VEC = 16 / sizeof(T);
+    const int lane = threadIdx.x & 31, sub = lane & (LP - 1);
+    const long long pix = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / LP;
+    const int head = (int)((uintptr_t)cost % 16 / sizeof(T));       // entries from the aligned address before
+    const long long end = head + (long long)npix * D;               // (entries counted from there)
+    const long long e0 = head + min(pix, (long long)npix - 1) * D;
+    const long long v0 = e0 / VEC;
+    const int nv = (int)((e0 + D - 1) / VEC - v0) + 1, shift = (int)(e0 - v0 * VEC);
+    const T* c = cost - head + v0 * VEC;                            // entry d is c[shift + d]
+    float best = -INFINITY;
+    int bd = 0x7FFFFFFF;
+    if (v0 * VEC < head || (v0 + nv) * VEC > end) {                 // at an end of the volume
+        for (int d0 = sub; d0 < D; d0 += LP * 4 * kWtaLoads) {
+            T t[4 * kWtaLoads];
+#pragma unroll
+            for (int k = 0; k < 4 * kWtaLoads; ++k)
+                if (d0 + k * LP < D) t[k] = c[shift + d0 + k * LP];
+#pragma unroll
+            for (int k = 0; k < 4 * kWtaLoads; ++k)
+                if (d0 + k * LP < D && (float)t[k] > best) { best = (float)t[k]; bd = d0 + k * LP; }
+        }
+    } else {
+        struct alignas(16) Vec { T v[VEC]; };
+        for (int k0 = sub; k0 < nv; k0 += LP * kWtaLoads) {
+            Vec t[kWtaLoads];
+#pragma unroll
+            for (int k = 0; k < kWtaLoads; ++k)
+                if (k0 + k * LP < nv) t[k] = *reinterpret_cast<const Vec*>(c + (k0 + k * LP) * VEC);
+#pragma unroll
+            for (int k = 0; k < kWtaLoads; ++k) {
+                const int at = k0 + k * LP, d = at * VEC - shift;
+                if (at == 0 || at == nv - 1) {
+#pragma unroll
+                    for (int j = 0; j < VEC; ++j) {
+                        const float v = (float)t[k].v[j];
+                        if ((unsigned)(d + j) < (unsigned)D && v > best) { best = v; bd = d + j; }
+                    }
+                } else if (at < nv) {
+#pragma unroll
+                    for (int j = 0; j < VEC; ++j) {
+                        const float v = (float)t[k].v[j];
+                        if (v > best) { best = v; bd = d + j; }
+                    }
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int off = LP / 2; off > 0; off >>= 1) {
+        const float ob = __shfl_xor_sync(kFull, best, off);
+        const int od = __shfl_xor_sync(kFull, bd, off);
+        if (ob > best || (ob == best && od < bd)) { best = ob; bd = od; }
+    }
+    if (sub == 0 && pix < npix) disp[pix] = (uint16_t)(bd == 0x7FFFFFFF ? 0 : bd);
+}
+
+template <typename T, int VEC, int LP>
+static void wta_aligned(const T* cost, int npix, int D, uint16_t* disp, cudaStream_t st) {
+    k_wta_volume<T, VEC, LP><<<(int)(((long long)npix * LP + 255) / 256), 256, 0, st>>>(cost, npix, D, disp);
+}
+template <typename T, int LP>
+static void wta_any(const T* cost, int npix, int D, uint16_t* disp, cudaStream_t st) {
+    k_wta_volume_any<T, LP><<<(int)(((long long)npix * LP + 255) / 256), 256, 0, st>>>(cost, npix, D, disp);
+}
+
+// Lanes per pixel. Aligned pixels: enough that each lane has about kWtaLoads loads, so that the
+// shuffle rounds serve many entries and no load slot stays empty. Others: up to three rounds of
+// loads per lane, since the pixels of a warp share the branch for the first and last vector; one
+// round in volumes of less than a million entries, which are a matter of latency (272x67, D = 42:
+// 3.6 us against 4.1).
+// Short pixels are read in narrower loads that they are aligned to: there the vectors of
+// k_wta_volume_any are mostly neighbours' (1920x1080 F16, D = 20 21 us against 37, D = 14 29 against
+// 37, D = 5 17 against 27; D = 17 58 against 37).
+template <typename T>
 static void wta_volume(const T* cost, int npix, int D, uint16_t* disp, cudaStream_t st) {
-    const int loads = D / VEC;
-    const int lp = loads <= 2 * kWtaLoads ? 2 : loads <= 4 * kWtaLoads ? 4 : loads <= 8 * kWtaLoads ? 8
-                   : loads <= 16 * kWtaLoads ? 16 : 32;
-    const int blocks = (int)(((long long)npix * lp + 255) / 256);
-    switch (lp) {
-        case 2: k_wta_volume<T, VEC, 2><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
-        case 4: k_wta_volume<T, VEC, 4><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
-        case 8: k_wta_volume<T, VEC, 8><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
-        case 16: k_wta_volume<T, VEC, 16><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
-        default: k_wta_volume<T, VEC, 32><<<blocks, 256, 0, st>>>(cost, npix, D, disp); break;
+    constexpr int VEC = 16 / sizeof(T);
+    const uintptr_t p = (uintptr_t)cost;
+    constexpr int shorts = 2 * kWtaLoads;
+    if (D % VEC == 0 && p % 16 == 0) {
+        const int loads = D / VEC;
+        if (loads <= shorts) wta_aligned<T, VEC, 2>(cost, npix, D, disp, st);
+        else if (loads <= 4 * kWtaLoads) wta_aligned<T, VEC, 4>(cost, npix, D, disp, st);
+        else if (loads <= 8 * kWtaLoads) wta_aligned<T, VEC, 8>(cost, npix, D, disp, st);
+        else if (loads <= 16 * kWtaLoads) wta_aligned<T, VEC, 16>(cost, npix, D, disp, st);
+        else wta_aligned<T, VEC, 32>(cost, npix, D, disp, st);
+    } else if (D % (VEC / 2) == 0 && p % 8 == 0 && D / (VEC / 2) <= shorts) {
+        wta_aligned<T, VEC / 2, 2>(cost, npix, D, disp, st);
+    } else if (D <= shorts) {
+        wta_aligned<T, 1, 2>(cost, npix, D, disp, st);
+    } else if (D <= 2 * shorts) {
+        wta_aligned<T, 1, 4>(cost, npix, D, disp, st);
+    } else {
+        const int loads = (D + VEC - 2) / VEC + 1;                  // the most of a pixel
+        const int per_lane = ((long long)npix * D < (1 << 20) ? 1 : 3) * kWtaLoads;
+        if (loads <= 2 * per_lane) wta_any<T, 2>(cost, npix, D, disp, st);
+        else if (loads <= 4 * per_lane) wta_any<T, 4>(cost, npix, D, disp, st);
+        else if (loads <= 8 * per_lane) wta_any<T, 8>(cost, npix, D, disp, st);
+        else wta_any<T, 16>(cost, npix, D, disp, st);
     }
 }
 
-// The widest load that every pixel's entries allow (base address and D): 16 or 8 bytes, else
-// one entry at a time.
 cudaError_t launch_wta_volume(const void* cost, int dtype, int W, int H, int D, uint16_t* disp,
                               cudaStream_t st) {
-    const int npix = W * H;
-    const uintptr_t p = (uintptr_t)cost;
-    if (dtype == 0) {
-        const float* c = (const float*)cost;
-        if (D % 4 == 0 && p % 16 == 0) wta_volume<float, 4>(c, npix, D, disp, st);
-        else if (D % 2 == 0 && p % 8 == 0) wta_volume<float, 2>(c, npix, D, disp, st);
-        else wta_volume<float, 1>(c, npix, D, disp, st);
-    } else {
-        const __half* c = (const __half*)cost;
-        if (D % 8 == 0 && p % 16 == 0) wta_volume<__half, 8>(c, npix, D, disp, st);
-        else if (D % 4 == 0 && p % 8 == 0) wta_volume<__half, 4>(c, npix, D, disp, st);
-        else wta_volume<__half, 1>(c, npix, D, disp, st);
-    }
+    if (dtype == 0) wta_volume((const float*)cost, W * H, D, disp, st);
+    else wta_volume((const __half*)cost, W * H, D, disp, st);
     return cudaGetLastError();
 }
 

@@ -71,3 +71,27 @@ def test_wta_loads_ties_and_special_values(d, off, dtype):
     n = np.where(np.isnan(v), -np.inf, v)
     ref = np.where(n.max(-1) == -np.inf, 0, n.argmax(-1))            # argmax: the smallest d of a tie
     assert np.array_equal(disp.cpu().numpy(), ref)
+
+
+# pixels that start at every place of a 16-byte vector, around the lanes per pixel (24, 48 and 96
+# vectors) and the short pixels; the volume's first and last pixels share vectors with what lies
+# around it, which must not count
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("d,off", [(5, 1), (9, 0), (12, 0), (14, 2), (15, 0), (16, 1), (17, 0), (20, 0), (28, 1), (34, 0), (93, 0), (95, 1), (97, 3),
+                                   (155, 0), (186, 2), (190, 0), (193, 5), (255, 0), (379, 0), (385, 7), (765, 1), (1019, 3)])
+def test_wta_of_pixels_off_16_bytes(d, off, dtype):
+    w, h = 41, 3
+    rng = np.random.default_rng(11 * d + off)
+    tdt, flag = (torch.float32, Z.ZNCC_F32) if dtype == "f32" else (torch.float16, Z.ZNCC_F16)
+    v = rng.integers(-40, 41, (h, w, d)).astype(np.float32)
+    v[0, :, d - 1] = 50.0                                            # the best at either end of a pixel
+    v[1, :, 0] = 50.0
+    v[2, ::2] = -60.0
+    buf = torch.full((16 + off + h * w * d + 16,), 99.0, dtype=tdt, device="cuda")
+    cost = buf[16 + off:16 + off + h * w * d].view(h, w, d)
+    cost.copy_(torch.from_numpy(v))
+    disp = torch.empty((h, w), dtype=torch.int16, device="cuda")
+    with Z.ZnccContext(w, h, d, 3) as ctx:
+        ctx.wta_disparity(cost, disp, flag)
+        torch.cuda.synchronize()
+    assert np.array_equal(disp.cpu().numpy(), v.argmax(-1))
