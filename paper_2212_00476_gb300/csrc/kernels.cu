@@ -231,24 +231,36 @@ __global__ void k_window_stats_row(const uint8_t* __restrict__ img, int pitch, i
     }
 }
 
-// Below this many pixel reads (centres x rows of the window) the row kernel is faster (us, row
-// kernel and k_window_stats, back to back: 206x179 9x9, 0.3 M reads, 4.6 and 8.3; 514x687 9x9,
-// 3.2 M, 6.5 and 10.7; 653x482 13x13, 4.1 M, 8.3 and 10.5; 816x981 7x7, 5.6 M, 10.5 and 8.4;
-// 752x733 13x13, 7.2 M, 10.4 and 8.5; 1840x754 11x11, 15 M, 16.7 and 10.5).
-constexpr long long kStatsRowReads = 5000000;
+// Whether k_window_stats is faster than one block per row, by the pixel reads of the latter (centres
+// x rows of the window). Us, row kernel and k_window_stats, back to back:
+//  - rows that start on 4 bytes, from 5 M reads on: 206x179 9x9, 0.3 M, 4.6 and 8.3; 514x687 9x9,
+//    3.2 M, 6.5 and 10.7; 653x482 13x13, 4.1 M, 8.3 and 10.5; 816x981 7x7, 5.6 M, 10.5 and 8.4;
+//    752x733 13x13, 7.2 M, 10.4 and 8.5; 1920x1080 3x3, 6.2 M, 14.6 and 10.4.
+//  - other rows, which it loads byte by byte: windows of nine rows and more, from 6.5 M reads on where
+//    its blocks of about 500 columns are mostly full (1241x375 15x15, 7.0 M, 11.3 and 10.5; 1277x717
+//    9x9, 8.2 M, 12.5 and 11.1), from 10 M on else (750x733 13x13, 7.1 M, 10.4 and 12.6; 749x833 15x15,
+//    9.4 M, 12.5 and 12.6; 1331x900 9x9, 10.8 M, 14.5 and 14.2; 1919x1080 11x11, 23 M, 24.8 and
+//    18.7). Small windows stay with the row kernel (1901x1000 3x3, 5.7 M, 12.6 and 18.7; 3001x2001
+//    7x7, 42 M, 43.4 and 45.8). Two word loads and a shift in place of the bytes were slower
+//    (1919x1080 11x11 24.8).
+static bool stats_tiles(int nx, int H, int r, bool words) {
+    const long long reads = (long long)nx * H * (2 * r + 1);
+    if (words) return reads >= 5000000;
+    return r >= 4 && reads >= (nx >= 1200 ? 6500000 : 10000000);
+}
 
 cudaError_t launch_window_stats(const uint8_t* img, int pitch, int W, int H, int r, int x_begin,
                                 int nx, int* S, int* Q, float* isig, int2* packed, cudaStream_t st) {
-    if ((long long)nx * H * (2 * r + 1) < kStatsRowReads) {
+    // four pixels a load where the rows start on 4 bytes; four results a store where every
+    // output row starts on 16
+    const int words = (uintptr_t)img % 4 == 0 && pitch % 4 == 0;
+    const int vec = nx % 4 == 0 && (uintptr_t)S % 16 == 0 && (uintptr_t)Q % 16 == 0 && (uintptr_t)isig % 16 == 0;
+    if (!stats_tiles(nx, H, r, words != 0)) {
         const size_t smem = 2 * sizeof(int) * (size_t)(nx + 2 * r);
         k_window_stats_row<<<H, 256, smem, st>>>(img, pitch, W, H, r, x_begin, nx, S, Q, isig, packed);
         return cudaGetLastError();
     }
     const dim3 grid((nx + stats_centres(r) - 1) / stats_centres(r), (H + kStatsRows - 1) / kStatsRows);
-    // four pixels a load where the rows start on 4 bytes; four results a store where every
-    // output row starts on 16
-    const int words = (uintptr_t)img % 4 == 0 && pitch % 4 == 0;
-    const int vec = nx % 4 == 0 && (uintptr_t)S % 16 == 0 && (uintptr_t)Q % 16 == 0 && (uintptr_t)isig % 16 == 0;
 #define ZNCC_STATS(R)                                                                                        \
     case R:                                                                                                  \
         k_window_stats<R><<<grid, kStatsThreads, 0, st>>>(img, pitch, W, H, x_begin, nx, words, vec, S, Q, isig, \

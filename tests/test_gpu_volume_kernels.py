@@ -95,3 +95,27 @@ def test_wta_of_pixels_off_16_bytes(d, off, dtype):
         ctx.wta_disparity(cost, disp, flag)
         torch.cuda.synchronize()
     assert np.array_equal(disp.cpu().numpy(), v.argmax(-1))
+
+
+# radii 3 and 6, rows off 4 bytes on both sides of the sizes from which they walk down the rows too
+@pytest.mark.parametrize("w,h,r,off,pad", [
+    (1004, 801, 3, 0, 0), (700, 601, 6, 0, 0), (1202, 449, 6, 0, 0), (1201, 660, 6, 2, 2), (1199, 700, 6, 1, 2),
+    (1241, 375, 7, 0, 0), (1003, 1111, 4, 3, 0), (1666, 1000, 1, 0, 0), (1001, 1500, 3, 0, 0)])
+def test_window_stats_of_large_images_radii_and_rows_off_4_bytes(w, h, r, off, pad):
+    test_window_stats_tiles_and_alignment(w, h, r, off, pad)
+
+
+# the kernels that read packed statistics of left centres and of right centres down to 1 - D, at
+# sizes where both statistics are computed down the rows (5 M reads, 4-byte rows): equal to the
+# costs of the kernel that computes its own statistics
+@pytest.mark.parametrize("w,h,d,r", [(1920, 600, 8, 2), (1920, 600, 9, 2), (1920, 600, 10, 2), (1920, 600, 11, 2), (1664, 450, 32, 4)])
+def test_packed_statistics_of_large_images(w, h, d, r):
+    rng = np.random.default_rng(w + d)
+    left, right = (torch.from_numpy(rng.integers(0, 256, (h, w), dtype=np.uint8)).cuda() for _ in range(2))
+    with Z.ZnccContext(w, h, d, 2 * r + 1) as ctx:
+        want, scan = (torch.empty((h, w, d), dtype=torch.float32, device="cuda") for _ in range(2))
+        ctx.zncc_cost_volume(left, right, want)
+        ctx.zncc_cost_volume_scan(left, right, scan)
+        assert torch.equal(scan, want)
+        ctx.zncc_cost_volume_mma(left, right, scan)
+        assert torch.equal(scan, want)
