@@ -408,6 +408,19 @@ zncc_status zncc_profile_read(zncc_ctx* ctx, double* total_ms, uint64_t* launche
 int zncc_profile_nkinds(void);
 const char* zncc_profile_kind_name(int kind);
 
+/* (tests) The last launch of kernel kind k on this context, host values out[0 .. n-1], n <= 7:
+ * variant (0 none yet; cost kernels 1 or 2: blocks per SM; DT pairs 1: the general line
+ * kernel, 2: the one of slabs and aligned volumes), blocks, threads, lanes per 16-position
+ * chunk, lines per block, columns that share warps, 1 where one chunk carries through the scan
+ * groups. A batch's launches are noted on its first context. Other kinds stay 0. */
+zncc_status zncc_launch_shape(zncc_ctx* ctx, int kind, int32_t* out, int n);
+
+/* (tests) Copies the intermediate volume of the context's last zncc_run (iters >= 1, not
+ * plane-resident) as its last stored pass pair left it: device [H][W][D] of the run's storage
+ * type (F16 values are divided by A_hat, I8 entries are FastDT codes). On the context's
+ * stream. ZNCC_EINVAL without such a run of that type. */
+zncc_status zncc_stored_volume(zncc_ctx* ctx, void* out, zncc_dtype dtype);
+
 #ifdef __cplusplus
 }
 #endif

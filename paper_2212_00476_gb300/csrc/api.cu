@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <initializer_list>
 #include <mutex>
 #include <new>
 #include <string>
@@ -95,6 +96,8 @@ struct zncc_ctx {
     void* vol = nullptr;          // the fused path's intermediate volume (on first use)
     size_t vol_bytes = 0;
     bool compact = false;         // the volume's pixels are padded to 4 entries, not to whole slabs
+    int vol_dtype = -1, vol_shift = 0;    // the last fused run's storage type (-1: no volume) and layout:
+    long long vol_dstride = 0;            // [slab][H][W][vol_dstride], 2^vol_shift disparities per slab
     float* ahat = nullptr;        // [nahat][H][W] DT responses of an all-ones plane (F16, I8 storage)
     float2* mulmap = nullptr;     // [nmul] maps of the pairs from 2 (F16) or 1 (I8) on:
     int nahat = 0, nmul = 0;      //        (A_hat_{p-1}, s2 / A_hat_p), line-major
@@ -132,6 +135,7 @@ struct zncc_ctx {
     std::vector<cudaEvent_t> events;
     int events_used = 0;
     std::vector<ProfRecord> records;
+    int32_t shapes[K_NKINDS][7] = {};     // zncc_launch_shape
     // zncc_run_host replayed as a CUDA graph: the arguments of the last call and of the captured
     // one, and the instantiated graph; gen counts changes of tuning and stream
     struct HostKey {
@@ -200,6 +204,10 @@ int prof_event(zncc_ctx* c) {
             (c)->records.push_back(ProfRecord{(kind), ev0_, ev1_});           \
         }                                                                     \
     } while (0)
+
+void note_shape(zncc_ctx* c, int kind, std::initializer_list<int32_t> shape) {
+    std::copy(shape.begin(), shape.end(), c->shapes[kind]);
+}
 
 // The chunk count is padded so that a line's threads fill whole warps (every warp-wide
 // shuffle then has all 32 lanes); padded chunks lie past the line end and hold zeros.
@@ -485,6 +493,7 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
             return fail(lc, ZNCC_EUNSUPPORTED, "the cost kernel's row band does not fit in shared memory");
         ZNCC_CUDA(lc, occupancy(two), "occupancy query");
         b.grid = std::max(1, std::min(b.total_items, std::max(1, lc->num_sms - reserve_sms) * std::max(1, bps)));
+        note_shape(lc, kind, {two ? 2 : 1, b.grid, threads, tq0, 1, 1, 0});
         ZNCC_LAUNCH(lc, kind, launch_zncc_row(r, b, threads, smem, mode, dtype, lc->cur), what);
     }
     return ZNCC_OK;
@@ -868,6 +877,7 @@ zncc_status run_dt_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* pa
         // steps, 709 and 636; 1920x1080x64, 28 steps, 182 and 175; 1800x400x128, 21 steps, 123 and
         // 130; 1600x1080x256, 13 warps, 546 and 572); columns lose by it.
         b.s.chain = s.horiz && b.s.nwl >= 14 && b.total_steps >= 24 * b.grid;
+        note_shape(lc, kind, {2, b.grid, threads, s.lanes, s.lines, s.cols, b.s.chain});
         ZNCC_LAUNCH(lc, kind, (dtype == 0 ? launch_dt_lines_f32 : launch_dt_lines_f16)(b, smem, mode, lc->cur), "DT pass pair");
     }
     return ZNCC_OK;
@@ -972,6 +982,7 @@ zncc_status run_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* passe
                 b.grid = two;
             }
         }
+        note_shape(lc, kind, {1, b.grid, threads, a0.tq, a0.lpc, 1, 0});
         ZNCC_LAUNCH(lc, kind, launch_line_batch(b, threads, smem, mode, dtype, lc->cur), "DT pass pair");
     }
     return ZNCC_OK;
@@ -1158,6 +1169,7 @@ zncc_status run_plane(zncc_ctx* lc, const PairIO* io, int n, float sigma_s, floa
 
 zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigma_r, int iters,
                       int storage) {
+    for (int i = 0; i < n; ++i) io[i].c->vol_dtype = -1;
     if (iters == 0) return run_rows(lc, io, n, kModeWta, 0, 0.0f, 0.0f, 0.0f, K_ZNCC_WTA, 0, "ZNCC + WTA");
     if (storage == ZNCC_F32) {      // pairs whose planes fit on chip take the plane-resident path
         PairIO plane[kMaxBatch];
@@ -1182,6 +1194,9 @@ zncc_status run_fused(zncc_ctx* lc, PairIO* io, int n, float sigma_s, float sigm
     for (int i = 0; i < n; ++i) {
         if (slabs) io[i].sd_shift = slab_shift(dt);
         io[i].dstride = slabs ? 1 << io[i].sd_shift : compact_entries(io[i].c->D);
+        io[i].c->vol_dtype = dt;
+        io[i].c->vol_shift = io[i].sd_shift;
+        io[i].c->vol_dstride = io[i].dstride;
     }
     const float K = (float)exp(-1.0 / (double)sigma_s);
     const float inv_sr255 = (float)(1.0 / (255.0 * (double)sigma_r));
@@ -1945,6 +1960,28 @@ zncc_status zncc_profile_read(zncc_ctx* c, double* total_ms, uint64_t* launches,
 }
 
 int zncc_profile_nkinds(void) { return K_NKINDS; }
+
+zncc_status zncc_launch_shape(zncc_ctx* c, int kind, int32_t* out, int n) {
+    if (!c || kind < 0 || kind >= K_NKINDS || !out || n < 0 || n > 7) return ZNCC_EINVAL;
+    std::copy(c->shapes[kind], c->shapes[kind] + n, out);
+    return ZNCC_OK;
+}
+
+zncc_status zncc_stored_volume(zncc_ctx* c, void* out, zncc_dtype dtype) {
+    if (!c) return ZNCC_EINVAL;
+    c->err.clear();
+    if (!out) return fail(c, ZNCC_EINVAL, "output pointer is NULL");
+    if (c->vol_dtype != (int)dtype) return fail(c, ZNCC_EINVAL, "no fused run has stored a volume of this type");
+    const size_t elem = volume_entry_bytes(c->vol_dtype), npix = (size_t)c->W * c->H;
+    const int per_slab = std::min(c->D, 1 << c->vol_shift);
+    for (int d = 0; d < c->D; d += per_slab) {
+        const char* slab = (const char*)c->vol + (d >> c->vol_shift) * npix * c->vol_dstride * elem;
+        ZNCC_CUDA(c, cudaMemcpy2DAsync((char*)out + d * elem, c->D * elem, slab, c->vol_dstride * elem,
+                                       std::min(per_slab, c->D - d) * elem, npix, cudaMemcpyDeviceToDevice,
+                                       c->stream), "volume copy");
+    }
+    return ZNCC_OK;
+}
 
 const char* zncc_profile_kind_name(int kind) {
     return kind >= 0 && kind < K_NKINDS ? kKindNames[kind] : nullptr;

@@ -71,6 +71,8 @@ SIGNATURES = [
                                ctypes.POINTER(ctypes.c_uint64), _i]),
     ("zncc_profile_nkinds", _i, []),
     ("zncc_profile_kind_name", ctypes.c_char_p, [_i]),
+    ("zncc_launch_shape", _i, [_vp, _i, ctypes.POINTER(ctypes.c_int32), _i]),
+    ("zncc_stored_volume", _i, [_vp, _vp, _i]),
 ]
 
 _lib = None
@@ -329,6 +331,18 @@ class ZnccContext:
         self._check(L.zncc_profile_read(self._h, ms, cnt, n))
         return {L.zncc_profile_kind_name(k).decode(): (ms[k], int(cnt[k])) for k in range(n)
                 if cnt[k]}
+
+    def launch_shape(self, kind: str) -> dict:
+        """The last launch of a kernel kind on this context (zncc_launch_shape)."""
+        L = lib()
+        k = [L.zncc_profile_kind_name(i).decode() for i in range(L.zncc_profile_nkinds())].index(kind)
+        out = (ctypes.c_int32 * 7)()
+        self._check(L.zncc_launch_shape(self._h, k, out, 7))
+        return dict(zip(("variant", "blocks", "threads", "lanes", "lines", "columns", "chain"), out))
+
+    def stored_volume(self, out, dtype: int = ZNCC_F32):
+        """The intermediate volume of the last zncc_run, [H][W][D], into out (a device tensor)."""
+        self._check(lib().zncc_stored_volume(self._h, _ptr(out), dtype))
 
     # -- the C calls --------------------------------------------------------------------
     def zncc_window_stats(self, img, S=None, Q=None, inv_sigma=None):
