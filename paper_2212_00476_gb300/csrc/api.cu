@@ -875,8 +875,10 @@ zncc_status run_dt_lines(zncc_ctx* lc, zncc_ctx* const* ctxs, const LinePass* pa
         // One chunk's lanes carry through the scan groups of long F32 rows (14 warps and more, W >
         // 1664) that a block has many steps of (us a pass without and with it: 1920x1080x256, 106
         // steps, 709 and 636; 1920x1080x64, 28 steps, 182 and 175; 1800x400x128, 21 steps, 123 and
-        // 130; 1600x1080x256, 13 warps, 546 and 572); columns lose by it.
-        b.s.chain = s.horiz && b.s.nwl >= 14 && b.total_steps >= 24 * b.grid;
+        // 130; 1600x1080x256, 13 warps, 546 and 572); columns lose by it, and F16 rows (a run of
+        // 1000x1000x256, 16 warps, 1402 and 1470; of 1900x300x256 979 and 988). F32 rows of eight
+        // lanes (dt_aggregate, W > 832) are level.
+        b.s.chain = dtype == 0 && s.horiz && b.s.nwl >= 14 && b.total_steps >= 24 * b.grid;
         note_shape(lc, kind, {2, b.grid, threads, s.lanes, s.lines, s.cols, b.s.chain});
         ZNCC_LAUNCH(lc, kind, (dtype == 0 ? launch_dt_lines_f32 : launch_dt_lines_f16)(b, smem, mode, lc->cur), "DT pass pair");
     }

@@ -49,6 +49,8 @@ def shape_of(launch):
     ("f16", 64, 50, 20, (8, 1, 1, 0), (8, 4, 1, 0), (8, 4, 1, 0)),
     ("f16", 1242, 375, 33, (8, 1, 1, 0), (8, 3, 1, 0), (8, 3, 1, 0)),
     ("f16", 1000, 500, 128, (8, 1, 1, 0), (8, 2, 1, 0), (8, 2, 1, 0)),
+    ("f16", 1000, 260, 800, (8, 1, 1, 0), (8, 4, 1, 0), (8, 4, 1, 0)),
+    ("f16", 1700, 80, 800, (4, 1, 1, 0), (8, 4, 1, 0), (8, 4, 1, 0)),
     ("f16", 2049, 20, 40, (4, 1, 1, 0), (8, 4, 1, 0), (8, 4, 1, 0)),
     ("f16", 3072, 12, 20, (2, 1, 1, 0), (8, 4, 1, 0), (8, 4, 1, 0)),
     ("f16", 40, 2000, 24, (8, 1, 1, 0), (4, 1, 1, 0), (4, 1, 1, 0)),
