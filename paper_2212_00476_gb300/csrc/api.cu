@@ -493,6 +493,17 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
             return fail(lc, ZNCC_EUNSUPPORTED, "the cost kernel's row band does not fit in shared memory");
         ZNCC_CUDA(lc, occupancy(two), "occupancy query");
         b.grid = std::max(1, std::min(b.total_items, std::max(1, lc->num_sms - reserve_sms) * std::max(1, bps)));
+        if (dtype == 2 && b.grid <= lc->num_sms) {
+            // A FastDT visit that starts past slice 0 computes it again: where that gives a block as
+            // many units as a whole row has, the blocks take whole rows (1900x120, D = 33, three
+            // slices, one iteration: 79 us a run, 91 split over all SMs; 1000x100, D = 96: 64 and 66)
+            const RowArgs& a = b.p[0];
+            const int slices = (a.D + kG * tq0 - 1) / (kG * tq0);
+            bool same = true;
+            for (int i = 1; i < b.npairs; ++i) same = same && b.p[i].nitems / b.p[i].H == slices;
+            const int rows = b.total_items / slices;
+            if (same && rows < b.grid && slices <= (b.total_items + b.grid - 1) / b.grid + 1) b.grid = rows;
+        }
         note_shape(lc, kind, {two ? 2 : 1, b.grid, threads, tq0, 1, 1, 0});
         ZNCC_LAUNCH(lc, kind, launch_zncc_row(r, b, threads, smem, mode, dtype, lc->cur), what);
     }

@@ -14,6 +14,19 @@ pytestmark = pytest.mark.gpu
 from paper_2212_00476_gb300 import zncc as Z  # noqa: E402
 
 
+# whole rows where a split would compute as many slices a block (three of a row; two and slice 0 again)
+@pytest.mark.parametrize("w,h,d,blocks", [(1900, 120, 33, 120), (1000, 100, 96, 100), (1900, 120, 16, 120)])
+def test_i8_rows_are_not_split_for_nothing(w, h, d, blocks):
+    p = make_pair(h, w, d, seed=w + d)
+    left, right = dev(p.left), dev(p.right)
+    disp = torch.full((h, w), -1, dtype=torch.int16, device="cuda")
+    with Z.ZnccContext(w, h, d, 9) as ctx:
+        ctx.zncc_run(left, right, disp, 20.0, 0.1, 1, Z.ZNCC_I8)
+        torch.cuda.synchronize()
+        assert ctx.launch_shape("zncc_cost_hpair")["blocks"] == blocks
+    check_against_oracle(p, disp.cpu().numpy().view(np.uint16), d, 9, 1, Z.ZNCC_I8)
+
+
 # (rows enough for four units per SM: the two-block layout is tried first)
 @pytest.mark.parametrize("w,d,win", [(2560, 1024, 3), (2560, 1024, 9), (2560, 1024, 15), (2305, 1000, 9), (2400, 784, 9)])
 def test_i8_rows_whose_padded_layout_does_not_fit(w, d, win):
