@@ -326,7 +326,8 @@ const char* zncc_status_string(zncc_status status);
 /* Launch-shape knobs of a context (0 = automatic for every key), for autotuning:
  *   ZNCC_TUNE_ROW_MINB2  cost kernel: 1 = the 96-register variant with two blocks per SM where the
  *                        block has at most 320 threads, 2 = one block per SM, 0 (automatic) = two
- *                        where every block gets at least two units (row, disparity slice) of work
+ *                        where both fit an SM and every block gets at least two units (row,
+ *                        disparity slice) of work; any other value as 1
  *   ZNCC_TUNE_ROW_SPB    cost kernel: disparity slices per block
  *   ZNCC_TUNE_H_TQ       horizontal DT pairs: lanes per 16-pixel chunk (2, 4 or 8)
  *   ZNCC_TUNE_V_TQ       vertical DT pairs: lanes per 16-pixel chunk (2, 4 or 8)

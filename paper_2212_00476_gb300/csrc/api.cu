@@ -1892,8 +1892,7 @@ zncc_status zncc_set_tuning(zncc_ctx* c, int key, int value) {
     if (value < 0) return fail(c, ZNCC_EINVAL, "tuning values are >= 0");
     switch (key) {
         case ZNCC_TUNE_ROW_MINB2:
-            if (value > 2) return fail(c, ZNCC_EINVAL, "blocks per SM of the cost kernel: 0, 1 (two) or 2 (one)");
-            c->row_minb2 = value;
+            c->row_minb2 = value > 2 ? 1 : value;       // (any other value: two, as 1)
             break;
         case ZNCC_TUNE_ROW_SPB: c->row_spb = value; break;
         case ZNCC_TUNE_AHAT_SMS: c->ahat_sms = value; break;

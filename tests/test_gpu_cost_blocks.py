@@ -14,6 +14,19 @@ pytestmark = pytest.mark.gpu
 from paper_2212_00476_gb300 import zncc as Z  # noqa: E402
 
 
+@pytest.mark.parametrize("value,blocks", [(1, 2), (2, 1), (3, 2), (100, 2)])
+def test_every_tuning_value_is_accepted(value, blocks):
+    p = make_pair(40, 200, 32, seed=3)
+    left, right = dev(p.left), dev(p.right)
+    disp = torch.empty((40, 200), dtype=torch.int16, device="cuda")
+    with Z.ZnccContext(200, 40, 32, 9) as ctx:
+        ctx.set_tuning(Z.ZNCC_TUNE_ROW_MINB2, value)
+        ctx.zncc_run(left, right, disp, 20.0, 0.1, 1, Z.ZNCC_F32)
+        torch.cuda.synchronize()
+        assert ctx.launch_shape("zncc_cost_hpair")["variant"] == blocks
+    check_against_oracle(p, disp.cpu().numpy().view(np.uint16), 32, 9, 1, Z.ZNCC_F32)
+
+
 # whole rows where a split would compute as many slices a block (three of a row; two and slice 0 again)
 @pytest.mark.parametrize("w,h,d,blocks", [(1900, 120, 33, 120), (1000, 100, 96, 100), (1900, 120, 16, 120)])
 def test_i8_rows_are_not_split_for_nothing(w, h, d, blocks):
