@@ -3,7 +3,8 @@
 For one problem shape (W, H, D, window, iterations, storage) it times the fused path with
 CUDA events for candidate values of each knob in turn (coordinate descent, a few rounds),
 keeps the fastest, and caches the result in a JSON file keyed by the shape, so that later
-runs apply it without searching:
+runs apply it without searching (an entry measured with other sources or other candidate values
+is not applied: the same setting may select another kernel there):
 
     from paper_2212_00476_gb300 import autotune
     best = autotune.tune(ctx, left, right, disp, sigma_s, sigma_r, iters, storage)
@@ -18,10 +19,12 @@ A_hat chain (whole chain before the first, or pass by pass).
 
 from __future__ import annotations
 
+import hashlib
 import json
 import os
 import threading
 
+from . import build as zbuild
 from . import zncc as Z
 
 CANDIDATES = {
@@ -44,6 +47,13 @@ _lock = threading.Lock()
 
 def shape_key(ctx, iters, storage):
     return f"{ctx.W}x{ctx.H}_D{ctx.D}_w{ctx.win}_it{iters}_s{storage}"
+
+
+def measured_with():
+    """What the cached timings depend on besides the shape: the library's sources and the
+    candidate values."""
+    values = sorted((NAMES[k], v) for k, v in CANDIDATES.items())
+    return hashlib.sha256(f"{zbuild._sources_digest()} {values}".encode()).hexdigest()[:16]
 
 
 def _load(path):
@@ -97,7 +107,7 @@ def tune(ctx, left, right, disp, sigma_s, sigma_r, iters, storage=Z.ZNCC_F32, re
     key = shape_key(ctx, iters, storage)
     with _lock:
         known = _load(cache)
-    if not force and key in known:
+    if not force and known.get(key, {}).get("measured_with") == measured_with():
         apply(ctx, known[key]["settings"])
         return known[key]
 
@@ -125,7 +135,7 @@ def tune(ctx, left, right, disp, sigma_s, sigma_r, iters, storage=Z.ZNCC_F32, re
         if not changed:
             break
     apply(ctx, settings)
-    result = {"settings": settings, "ms": best_ms}
+    result = {"settings": settings, "ms": best_ms, "measured_with": measured_with()}
     with _lock:
         known = _load(cache)
         known[key] = result

@@ -116,3 +116,25 @@ def test_results_are_cached_per_shape_and_reapplied(monkeypatch, tmp_path):
     m = len(timed)
     tune(FakeCtx(), path, force=True)           # force: searched again
     assert len(timed) > m
+
+
+def test_entries_measured_otherwise_are_not_applied(monkeypatch, tmp_path):
+    """Entries of other sources or candidate values, and of caches without that mark, are searched
+    again: the same setting may mean another kernel."""
+    timed = install_timer(monkeypatch, separable)
+    key = AT.shape_key(FakeCtx(), 3, Z.ZNCC_F32)
+    stale = {"settings": {**BEST, "line_loads": 1}, "ms": 0.1}
+    for i, mark in enumerate(({}, {"measured_with": "0" * 16})):
+        path = tmp_path / f"{i}.json"
+        path.write_text(json.dumps({key: {**stale, **mark}, "other": stale}))
+        n = len(timed)
+        assert tune(FakeCtx(), path)["settings"] == BEST and len(timed) > n
+        data = json.loads(path.read_text())
+        assert data[key]["settings"] == BEST and data["other"] == stale
+        n = len(timed)
+        tune(FakeCtx(), path)                   # its own entry is applied
+        assert len(timed) == n
+
+    mark = AT.measured_with()
+    monkeypatch.setitem(AT.CANDIDATES, Z.ZNCC_TUNE_ROW_MINB2, [0, 1])
+    assert AT.measured_with() != mark
