@@ -329,8 +329,12 @@ const char* zncc_status_string(zncc_status status);
  *                        where both fit an SM and every block gets at least two units (row,
  *                        disparity slice) of work; any other value as 1
  *   ZNCC_TUNE_ROW_SPB    cost kernel: disparity slices per block
- *   ZNCC_TUNE_H_TQ       horizontal DT pairs: lanes per 16-pixel chunk (2, 4 or 8)
- *   ZNCC_TUNE_V_TQ       vertical DT pairs: lanes per 16-pixel chunk (2, 4 or 8)
+ *   ZNCC_TUNE_H_TQ       horizontal DT pairs: lanes per 16-pixel chunk (2, 4 or 8) of the general
+ *                        line kernel. Passes in the slab kernel choose their lanes themselves and
+ *                        take 32 / value as the chunks per scan group, which decides the order in
+ *                        which carries are combined: the last bits of a map depend on it, as in
+ *                        the general kernel
+ *   ZNCC_TUNE_V_TQ       vertical DT pairs: the same
  *   ZNCC_TUNE_AHAT_SMS   (F16, I8 storage, ZNCC_TUNE_ROW_MINB2 = 1) SMs the cost kernel leaves
  *                        free for the A_hat chain, which runs beside it on a second stream
  *                        (default 8)
@@ -348,8 +352,9 @@ const char* zncc_status_string(zncc_status status);
  *                        TMA unit) where both images and the pitch are 16-byte aligned and W is
  *                        a multiple of 16, plain loads elsewhere
  *   ZNCC_TUNE_V_LPC      vertical DT pairs that store the volume: at most this many adjacent
- *                        columns per block (1, 2 or 4; 0 = automatic). Adjacent columns of a row share DRAM pages,
- *                        so wider groups make longer runs per page at the cost of residency;
+ *                        columns per block (1, 2 or 4; 0 = automatic). Adjacent columns of a row
+ *                        share DRAM pages, so wider groups make longer runs per page at the cost
+ *                        of residency;
  *                        the last vertical pair with WTA keeps the automatic shape
  *   ZNCC_TUNE_LINE_LOADS DT pairs: 0 (automatic) = the fused runs with F32 and F16 storage keep
  *                        their volume in slabs of 64 bytes per pixel and bring each step's

@@ -397,7 +397,9 @@ __device__ __forceinline__ float out_scale(float m) { return m; }
 // o[j] = fmaf(s, y[j], z[j]) and x[j] = s * x[j] for the four disparities of a position (o may
 // be y or z). PACKED: as two packed pairs (__ffma2_rn / __fmul2_rn, sm_100 and later), which
 // round each component exactly as fmaf and a single multiply do: the same bits in half the
-// floating-point instructions.
+// floating-point instructions. The DT line passes (15% fewer instructions there) and the cost
+// kernel's 96-register variant take them; in its 128-register variant the packed form measured
+// slower (117 -> 124 us at 1280x384x128), so that one keeps the scalar form.
 template <bool PACKED>
 __device__ __forceinline__ void fma4(float s, const float (&y)[4], const float (&z)[4], float (&o)[4]) {
     if constexpr (PACKED) {
@@ -423,10 +425,7 @@ __device__ __forceinline__ void mul4(float s, float (&x)[4]) {
     }
 }
 
-// PACKED: the sweeps, scans and carries use the packed pairs of fma4 / mul4 (the DT line
-// passes: 15% fewer instructions; in the cost kernel's fused pair the packed form measured
-// slower, 117 -> 124 us at 1280x384x128, so that one keeps the scalar form).
-template <bool SCALE = true, bool PACKED = false, typename Hook = NoHook, typename MulT = float2>
+template <bool SCALE = true, typename Hook = NoHook, typename MulT = float2>
 __device__ __forceinline__ void dt_pair(float (&v)[kL][4], const float4* __restrict__ co, int tq, int dq,
                                         int lane, int wl, int nwl, float* sa, float4* sb, float s2,
                                         const MulT* __restrict__ mul = nullptr,
@@ -442,7 +441,7 @@ __device__ __forceinline__ void dt_pair(float (&v)[kL][4], const float4* __restr
 #pragma unroll
         for (int i = 0; i < kL; ++i) {
             const float w = co[i].x;
-            fma4<PACKED>(w, u, v[i], u);
+            fma4<true>(w, u, v[i], u);
 #pragma unroll
             for (int j = 0; j < 4; ++j) v[i][j] = u[j];
         }
@@ -462,7 +461,7 @@ __device__ __forceinline__ void dt_pair(float (&v)[kL][4], const float4* __restr
 #pragma unroll
             for (int j = 0; j < 4; ++j) B2[j] = __shfl_up_sync(kFull, B[j], off);
             if (lane >= off) {
-                fma4<PACKED>(A, B2, B, B);
+                fma4<true>(A, B2, B, B);
                 A *= A2;
             }
         }
@@ -497,27 +496,18 @@ __device__ __forceinline__ void dt_pair(float (&v)[kL][4], const float4* __restr
             const float a2 = sa[w2 * tq + dq];
             const float4 b2 = sb[w2 * tq + dq];
             const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
-            fma4<PACKED>(a2, F, b4, F);
+            fma4<true>(a2, F, b4, F);
         }
-        fma4<PACKED>(Ae, F, Be, F);
+        fma4<true>(Ae, F, Be, F);
         float h[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int i = kL - 1; i >= 0; --i) {
             const float4 c = co[i];
-            if constexpr (PACKED) {
-                float ft[4];
-                fma4<true>(c.y, F, v[i], ft);
-                fma4<true>(c.z, h, ft, h);
+            float ft[4];
+            fma4<true>(c.y, F, v[i], ft);
+            fma4<true>(c.z, h, ft, h);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) v[i][j] = h[j];
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float ft = fmaf(c.y, F[j], v[i][j]);
-                    h[j] = fmaf(c.z, h[j], ft);
-                    v[i][j] = h[j];
-                }
-            }
+            for (int j = 0; j < 4; ++j) v[i][j] = h[j];
         }
         A = co[0].w;
 #pragma unroll
@@ -531,7 +521,7 @@ __device__ __forceinline__ void dt_pair(float (&v)[kL][4], const float4* __restr
 #pragma unroll
             for (int j = 0; j < 4; ++j) B2[j] = __shfl_down_sync(kFull, B[j], off);
             if (lane + off < 32) {
-                fma4<PACKED>(A, B2, B, B);
+                fma4<true>(A, B2, B, B);
                 A *= A2;
             }
         }
@@ -564,22 +554,22 @@ __device__ __forceinline__ void dt_pair(float (&v)[kL][4], const float4* __restr
             const float a2 = sa[(nwl + w2) * tq + dq];
             const float4 b2 = sb[(nwl + w2) * tq + dq];
             const float b4[4] = {b2.x, b2.y, b2.z, b2.w};
-            fma4<PACKED>(a2, G, b4, G);
+            fma4<true>(a2, G, b4, G);
         }
-        fma4<PACKED>(Ae, G, Be, G);
+        fma4<true>(Ae, G, Be, G);
         if (SCALE && (mul || s2 != 1.0f)) {
 #pragma unroll
             for (int i = 0; i < kL; ++i) {
                 const float b = co[i].w;
                 const float m = mul ? out_scale(mul[i]) : s2;
-                fma4<PACKED>(b, G, v[i], v[i]);
-                mul4<PACKED>(m, v[i]);
+                fma4<true>(b, G, v[i], v[i]);
+                mul4<true>(m, v[i]);
             }
         } else {                            // unscaled (s2 == 1: the caller runs the literal chain)
 #pragma unroll
             for (int i = 0; i < kL; ++i) {
                 const float b = co[i].w;
-                fma4<PACKED>(b, G, v[i], v[i]);
+                fma4<true>(b, G, v[i], v[i]);
             }
         }
     }

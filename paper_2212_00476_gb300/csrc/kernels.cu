@@ -849,7 +849,7 @@ __global__ void __launch_bounds__(512) k_line_pair(const __grid_constant__ LineB
             for (int i = 0; i < kL; ++i) mul4<true>(mul[i].x, v[i]);
         }
         // the staging buffer is free once the forward sweep has read it: refill it two ahead
-        dt_pair<MODE != kLineWta, true>(v, co, tq, dq, lane, rank * nwl + wl, nwl_all, sa, sb, a.s2, mul,
+        dt_pair<MODE != kLineWta>(v, co, tq, dq, lane, rank * nwl + wl, nwl_all, sa, sb, a.s2, mul,
                 [&]() {
                     prefetch(pf, n_s & 1);
                     advance(pf);

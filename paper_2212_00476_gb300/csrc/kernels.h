@@ -42,7 +42,8 @@ struct RowArgs {
     int bulk;                 // (HPair) stage the image rows by bulk asynchronous copies: both
                               // images and the pitch 16-byte aligned, W a multiple of 16
     int item0, nitems;        // this pair's units (row, slice), or rows (Wta), in a batched launch
-    int lpad;                 // spare entries (0, or 1 with minb2) per chunk of the left band and statistics
+    int lpad;                 // spare entries per chunk of the left band and statistics: 1, or 0 in the
+                              // one-block variant where a row would not fit with them
     // filled by zncc_row_layout: log2(tq), the planes of the cost arrays, and byte offsets in shared memory of the packed right
     // band, the window statistics, the coefficients, the scan buffers, FastDT's output scales and
     // references, and the guide row (bulk)
