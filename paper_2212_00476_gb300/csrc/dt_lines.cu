@@ -303,8 +303,12 @@ static const void* dt_lines_fn_t(int lanes, int cols) {
 }
 template <int NP>
 static const void* dt_lines_fn(int mode, int lanes, int cols, int threads) {
-    if (mode == kLineStore)
-        return threads <= 512 ? dt_lines_fn_t<kLineStore, NP, 512>(lanes, cols) : dt_lines_fn_t<kLineStore, NP, kDtThreads>(lanes, cols);
+    if (mode == kLineStore) {
+        if (threads <= 512) return dt_lines_fn_t<kLineStore, NP, 512>(lanes, cols);
+        // (F32 store passes take blocks of at most 512 threads: a larger one has no kernel)
+        if constexpr (std::is_same<DtElem, float>::value) return nullptr;
+        else return dt_lines_fn_t<kLineStore, NP, kDtThreads>(lanes, cols);
+    }
     return threads <= 512 ? dt_lines_fn_t<kLineWta, NP, 512>(lanes, cols) : dt_lines_fn_t<kLineWta, NP, kDtThreads>(lanes, cols);
 }
 
@@ -312,6 +316,7 @@ cudaError_t DT_NAME(dt_lines_occupancy)(int mode, const DtShape& s, int threads,
                                         int* blocks_per_sm) {
     const void* fn = single ? dt_lines_fn<1>(mode, s.lanes, s.cols, threads)
                             : dt_lines_fn<kMaxBatch>(mode, s.lanes, s.cols, threads);
+    if (!fn) return cudaErrorInvalidValue;
     cudaError_t e = set_max_smem(fn, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
@@ -325,6 +330,7 @@ cudaError_t DT_NAME(launch_dt_lines)(const DtBatch<kMaxBatch>& b, size_t smem, i
     const bool single = b.npairs == 1;
     const void* fn = single ? dt_lines_fn<1>(mode, b.s.lanes, b.s.cols, threads)
                             : dt_lines_fn<kMaxBatch>(mode, b.s.lanes, b.s.cols, threads);
+    if (!fn) return cudaErrorInvalidValue;
     cudaError_t e = set_max_smem(fn, smem);
     if (e != cudaSuccess) return e;
     if (!single) return launch_batch(cfg, fn, b);
