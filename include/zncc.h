@@ -424,7 +424,8 @@ zncc_status zncc_launch_shape(zncc_ctx* ctx, int kind, int32_t* out, int n);
 /* (tests) Copies the intermediate volume of the context's last zncc_run (iters >= 1, not
  * plane-resident) as its last stored pass pair left it: device [H][W][D] of the run's storage
  * type (F16 values are divided by A_hat, I8 entries are FastDT codes). On the context's
- * stream. ZNCC_EINVAL without such a run of that type. */
+ * stream. ZNCC_EINVAL without such a run of that type, or after a zncc_run_host that replayed
+ * a captured run. */
 zncc_status zncc_stored_volume(zncc_ctx* ctx, void* out, zncc_dtype dtype);
 
 #ifdef __cplusplus

@@ -1831,6 +1831,7 @@ zncc_status zncc_run_host(zncc_ctx* c, const uint8_t* left_host, const uint8_t* 
     const zncc_ctx::HostKey key{left_host, right_host, disp_host, dleft,         dright,      dmap,
                                 pitch,     iters,      (int)storage, sigma_s, sigma_r, c->gen};
     if (c->host_graph && map_pinned && imgs_pinned && key == c->host_key && !c->profiling) {
+        c->vol_dtype = -1;              // (the captured run's layout of the volume is not kept)
         ZNCC_CUDA(c, cudaGraphLaunch(c->host_graph, c->stream), "graph launch");
         ZNCC_CUDA(c, cudaStreamSynchronize(c->stream), "stream synchronize");
         return ZNCC_OK;

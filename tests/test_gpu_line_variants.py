@@ -101,3 +101,25 @@ def test_stored_volume_needs_a_run_of_that_type():
                 with pytest.raises(Z.ZnccError):
                     ctx.stored_volume(vol)
         torch.cuda.synchronize()
+
+
+def test_no_stored_volume_after_a_replayed_host_run():
+    """A replayed run writes the volume in the layout of its capture, not of the last direct run."""
+    w, h, d = 64, 32, 20
+    p = make_pair(h, w, d, seed=3)
+    left, right = dev(p.left), dev(p.right)
+    host = [torch.from_numpy(np.ascontiguousarray(a)).pin_memory() for a in (p.left, p.right)]
+    host.append(torch.zeros((h, w), dtype=torch.int16).pin_memory())
+    args = [host[0].numpy(), host[1].numpy(), host[2].numpy().view(np.uint16)]
+    disp = torch.empty((h, w), dtype=torch.int16, device="cuda")
+    vol = torch.empty((h, w, d), dtype=torch.float16, device="cuda")
+    with Z.ZnccContext(w, h, d, 5, stream=torch.cuda.Stream()) as ctx:
+        torch.cuda.synchronize()
+        ctx.zncc_run(left, right, disp, 20.0, 0.1, 2, Z.ZNCC_F16)
+        ctx.stored_volume(vol, Z.ZNCC_F16)
+        for _ in range(3):                  # issued, captured, replayed
+            ctx.zncc_run_host(*args, 20.0, 0.1, 2, Z.ZNCC_F32)
+        ctx.zncc_run(left, right, disp, 20.0, 0.1, 2, Z.ZNCC_F16)
+        ctx.zncc_run_host(*args, 20.0, 0.1, 2, Z.ZNCC_F32)
+        with pytest.raises(Z.ZnccError):
+            ctx.stored_volume(vol, Z.ZNCC_F16)
