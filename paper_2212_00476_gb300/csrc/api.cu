@@ -359,6 +359,11 @@ long long row_units(const zncc_ctx* c) {
     return (long long)c->H * ((c->D + ds - 1) / ds);
 }
 
+// A volume off the alignment of four entries has its lanes trade entries before the stores from four
+// disparities (below, one lane of a chunk holds them all) and this many entries on (zncc_row_item
+// has both sides measured). The two-blocks-per-SM variant always trades.
+constexpr long long kTradeEntries = 1 << 19;
+
 // Cost-kernel launches over the pairs (one per window radius among them). A block covers
 // one row and a run of disparity slices (the band of a block spans its slices, so the run
 // shrinks until the block fits in shared memory); in Wta mode a block covers every
@@ -423,6 +428,7 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
                 a.coefH_out = mode == kModeHPair ? c->coefH : nullptr;
                 a.s2 = s2;
                 a.minb2 = minb2 ? 1 : 0;
+                a.trade = c->D >= kG && (long long)c->W * c->H * c->D >= kTradeEntries ? 1 : 0;
                 a.wta.disp = pio.disp;
                 a.wta.first = 1;
                 a.wta.last = 1;
@@ -474,14 +480,16 @@ zncc_status run_rows(zncc_ctx* lc, const PairIO* io, int n, int mode, int dtype,
         //    which beyond L2 leave it like that (640x300, D = 1000 F16, 2000 bytes a pixel: 155 and
         //    181; 1280x384, D = 124: 113 and 132; F32, D = 400, 25 slices: 178 and 184, D = 256, 16
         //    slices: 126 and 121; in L2: 1280x720, D = 61 F16: 135 and 128).
-        // Not with WTA alone, whose rows are whole units and whose running best spills there.
+        // Not with WTA alone, whose rows are whole units and whose running best spills there, nor with
+        // fewer than four disparities off the alignment, which have nothing to trade (400x640, D = 2
+        // F32: 18.2 with one block and 22.9).
         bool two = nch0 * tq0 <= 320;
         if (two && !all_two) {
             const zncc_ctx* c = io[first].c;
             const long long row = (long long)c->D * (dtype == 0 ? 4 : 2);
             const bool scattered = mode == kModeRawAny ||
                                    (mode == kModeRaw && (row % 32 != 0 || (dtype == 0 && c->D > 20 * kG * tq0)));
-            two = !any_one && mode != kModeWta && units >= 4ll * lc->num_sms &&
+            two = !any_one && mode != kModeWta && units >= 4ll * lc->num_sms && !(mode == kModeRawAny && c->D < kG) &&
                   !(scattered && row * c->W * c->H > lc->l2_bytes);
         }
         two = two && fill(true);

@@ -42,6 +42,7 @@ struct RowArgs {
     int bulk;                 // (HPair) stage the image rows by bulk asynchronous copies: both
                               // images and the pitch 16-byte aligned, W a multiple of 16
     int item0, nitems;        // this pair's units (row, slice), or rows (Wta), in a batched launch
+    int trade;                // (RawAny) lanes trade entries before the stores; the two-block variant always does
     int lpad;                 // spare entries per chunk of the left band and statistics: 1, or 0 in the
                               // one-block variant where a row would not fit with them
     // filled by zncc_row_layout: log2(tq), the planes of the cost arrays, and byte offsets in shared memory of the packed right

@@ -399,29 +399,41 @@ __device__ __forceinline__ bool zncc_row_item(const RowArgs& a, int y, int s_beg
             // and a 32-byte sector is written in fewer pieces (us a call, every fourth entry and this:
             // 1280x384x127 F32 276 and 186, 1296x315x246 F16 414 and 258, 2500x700x61 F32 672 and 568).
             // (A block is whole warps, all of them here.)
-            const bool quad = tq >= 4;
-            const int l = dq & (quad ? 3 : 1);
-            const int left = a.d_hi - (d_first - 3 * l);     // entries from the first that this lane stores
-            T* p = q - 3 * l;
-            const int o2 = quad ? 8 : 2, o3 = o2 + 4;
+            // Small volumes (a.trade) are written from registers as they are: there the kernel is a matter of
+            // latency and of fetching its instructions (160x64x17 F32 6.7 and 5.4 us, 59x76x1 F16 7.6 and
+            // 6.3, 200x100x19 6.5 and 5.5; level at 160x100x33, 320x96x21 F16 6.7 and 7.6).
+            if (!PAD && !a.trade) {
+                if (nvalid > 0)
 #pragma unroll
-            for (int i = 0; i < kL; ++i) {
-                float e[4] = {v[i][0], v[i][1], v[i][2], v[i][3]};
-                const float r0 = __shfl_xor_sync(kFull, l & 1 ? e[0] : e[1], 1);
-                const float r1 = __shfl_xor_sync(kFull, l & 1 ? e[2] : e[3], 1);
-                if (l & 1) { e[0] = r0; e[2] = r1; } else { e[1] = r0; e[3] = r1; }
-                if (quad) {
-                    const float r2 = __shfl_xor_sync(kFull, l & 2 ? e[0] : e[2], 2);
-                    const float r3 = __shfl_xor_sync(kFull, l & 2 ? e[1] : e[3], 2);
-                    if (l & 2) { e[0] = r2; e[1] = r3; } else { e[2] = r2; e[3] = r3; }
+                    for (int i = 0; i < kL; ++i) {
+                        if (x0 + i < W) st4(q, nvalid, false, v[i]);
+                        q += a.dstride;
+                    }
+            } else {
+                const bool quad = tq >= 4;
+                const int l = dq & (quad ? 3 : 1);
+                const int left = a.d_hi - (d_first - 3 * l);     // entries from the first that this lane stores
+                T* p = q - 3 * l;
+                const int o2 = quad ? 8 : 2, o3 = o2 + 4;
+#pragma unroll
+                for (int i = 0; i < kL; ++i) {
+                    float e[4] = {v[i][0], v[i][1], v[i][2], v[i][3]};
+                    const float r0 = __shfl_xor_sync(kFull, l & 1 ? e[0] : e[1], 1);
+                    const float r1 = __shfl_xor_sync(kFull, l & 1 ? e[2] : e[3], 1);
+                    if (l & 1) { e[0] = r0; e[2] = r1; } else { e[1] = r0; e[3] = r1; }
+                    if (quad) {
+                        const float r2 = __shfl_xor_sync(kFull, l & 2 ? e[0] : e[2], 2);
+                        const float r3 = __shfl_xor_sync(kFull, l & 2 ? e[1] : e[3], 2);
+                        if (l & 2) { e[0] = r2; e[1] = r3; } else { e[2] = r2; e[3] = r3; }
+                    }
+                    if (x0 + i < W) {
+                        if (0 < left) st1(p, e[0]);
+                        if (4 < left) st1(p + 4, e[1]);
+                        if (o2 < left) st1(p + o2, e[2]);
+                        if (o3 < left) st1(p + o3, e[3]);
+                    }
+                    p += a.dstride;
                 }
-                if (x0 + i < W) {
-                    if (0 < left) st1(p, e[0]);
-                    if (4 < left) st1(p + 4, e[1]);
-                    if (o2 < left) st1(p + o2, e[2]);
-                    if (o3 < left) st1(p + o3, e[3]);
-                }
-                p += a.dstride;
             }
         } else if (nvalid > 0) {
             // (Raw: the costs are finished before the first store; interleaved, the addresses would

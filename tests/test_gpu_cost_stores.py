@@ -45,3 +45,15 @@ def test_stores_at_every_alignment(w, h, d, win, off, dtype):
     want = volume(left, right, (d + 3) // 4 * 4, win, dtype, 0, 0)[:, :, :d]
     for minb2 in (0, 1):
         assert torch.equal(volume(left, right, d, win, dtype, off, minb2), want)
+
+
+# volumes of more than half a million entries, whose lanes trade entries before the stores: blocks of
+# eight, four and two lanes per chunk, one and two per SM
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("w,h,d,win,off", [
+    (1024, 512, 1, 3, 0), (1023, 257, 2, 3, 1), (70, 420, 18, 9, 0), (641, 50, 17, 9, 3), (250, 70, 31, 9, 0),
+    (1025, 40, 15, 5, 0), (1300, 13, 33, 13, 1), (1999, 5, 54, 9, 0), (2049, 38, 7, 9, 0), (2500, 24, 9, 9, 1),
+    (3072, 8, 22, 15, 0), (600, 30, 32, 7, 2)])
+def test_stores_of_larger_volumes(w, h, d, win, off, dtype):
+    assert w * h * d >= 1 << 19
+    test_stores_at_every_alignment(w, h, d, win, off, dtype)
