@@ -358,13 +358,15 @@ const char* zncc_status_string(zncc_status status);
  *                        the last vertical pair with WTA keeps the automatic shape
  *   ZNCC_TUNE_LINE_LOADS DT pairs: 0 (automatic) = the fused runs with F32 and F16 storage keep
  *                        their volume in slabs of 64 bytes per pixel and bring each step's
- *                        16-position chunks into shared memory by TMA tensor copies; elsewhere
- *                        (I8 storage, dt_aggregate) one TMA copy per chunk and slice in the
- *                        horizontal pairs where the volume and its pixel stride are 16-byte
- *                        aligned, F32 or F16 reads span at most four chunks per shared-memory
- *                        wavefront, a line fits one CTA and shared memory allows, 16-byte cp.async
- *                        otherwise; 1 = the volume as [H][W][D], cp.async only; 2 = the volume as
- *                        [H][W][D], TMA in both directions. The maps do not depend on it
+ *                        16-position chunks into shared memory by TMA tensor copies, and
+ *                        dt_aggregate runs the same kernel on a volume whose pixels start on 16
+ *                        bytes where a chunk takes eight lanes; elsewhere (I8 storage, other
+ *                        volumes) one TMA copy per chunk and slice in the horizontal pairs where
+ *                        the volume and its pixel stride are 16-byte aligned, F32 or F16 reads
+ *                        span at most four chunks per shared-memory wavefront, a line fits one
+ *                        CTA and shared memory allows, 16-byte cp.async otherwise; 1 = the volume
+ *                        as [H][W][D], cp.async only; 2 = the volume as [H][W][D], TMA in both
+ *                        directions. The maps do not depend on it
  *   ZNCC_TUNE_WAIT_DRILL (tests) 1 = every DT pair launch has one thread per block wait, with a
  *                        64-poll limit, for an mbarrier phase that nothing completes; the wait
  *                        runs out and records fault bit 2 (see zncc_device_faults) while the

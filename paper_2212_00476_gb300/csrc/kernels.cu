@@ -70,7 +70,7 @@ void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, dim3 grid
 // 4-byte aligned. The row's column sums go through shared memory (two buffers, one barrier a
 // row) and each thread sums the windows of four adjacent centres from 16-byte reads.
 // Bound by latency and launch at these sizes (26 MB in all at 1920x1080); one block per row
-// with a byte load per pixel and window row took 25.0 us there, this 10.4.
+// with a byte load per pixel and window row took 25.2 us a call there, this 11.7.
 // S, Q exact int32; inv_sigma = rsqrtf(n Q - S^2) (within 2
 // ulp of 1/sqrt) or 0; the cost kernel computes its statistics the same way, bit for bit.
 // n Q - S^2 < 2^31 for every window side <= 15 (its maximum is n^2 * 127.5^2), so it is
