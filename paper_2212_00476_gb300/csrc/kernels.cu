@@ -1166,7 +1166,9 @@ static void wta_any(const T* cost, int npix, int D, uint16_t* disp, cudaStream_t
 // shuffle rounds serve many entries and no load slot stays empty. Others: up to three rounds of
 // loads per lane, since the pixels of a warp share the branch for the first and last vector; one
 // round in volumes of less than a million entries, which are a matter of latency (272x67, D = 42:
-// 3.6 us against 4.1).
+// 3.6 us against 4.1). Pixels of 97 to 192 vectors take eight lanes and up to six rounds: 16 lanes
+// leave their last round nearly empty (1500x586x541 F32 283 and 270 us, 784x117x577 38.9 and 36.9,
+// F16 784x87x777 24.9 and 20.5; above, 1500x408x777 F32 268 and 272, 1500x310x1021 262 and 273).
 // Short pixels are read in narrower loads that they are aligned to: there the vectors of
 // k_wta_volume_any are mostly neighbours' (1920x1080 F16, D = 20 21 us against 37, D = 14 29 against
 // 37, D = 5 17 against 27; D = 17 58 against 37).
@@ -1190,10 +1192,11 @@ static void wta_volume(const T* cost, int npix, int D, uint16_t* disp, cudaStrea
         wta_aligned<T, 1, 4>(cost, npix, D, disp, st);
     } else {
         const int loads = (D + VEC - 2) / VEC + 1;                  // the most of a pixel
-        const int per_lane = ((long long)npix * D < (1 << 20) ? 1 : 3) * kWtaLoads;
+        const bool small = (long long)npix * D < (1 << 20);
+        const int per_lane = (small ? 1 : 3) * kWtaLoads;
         if (loads <= 2 * per_lane) wta_any<T, 2>(cost, npix, D, disp, st);
         else if (loads <= 4 * per_lane) wta_any<T, 4>(cost, npix, D, disp, st);
-        else if (loads <= 8 * per_lane) wta_any<T, 8>(cost, npix, D, disp, st);
+        else if (loads <= (small ? 8 : 16) * per_lane) wta_any<T, 8>(cost, npix, D, disp, st);
         else wta_any<T, 16>(cost, npix, D, disp, st);
     }
 }

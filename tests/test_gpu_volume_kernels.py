@@ -119,3 +119,26 @@ def test_packed_statistics_of_large_images(w, h, d, r):
         assert torch.equal(scan, want)
         ctx.zncc_cost_volume_mma(left, right, scan)
         assert torch.equal(scan, want)
+
+
+# volumes of more than a million entries: pixels of one to six rounds of loads at eight lanes
+# (up to 192 vectors) and of 16 lanes
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("d,off", [(189, 1), (379, 3), (385, 0), (511, 2), (523, 0), (765, 1), (769, 0), (999, 2), (1021, 5)])
+def test_wta_of_large_volumes_off_16_bytes(d, off, dtype):
+    w = 41
+    h = (1 << 20) // (w * d) + 1
+    rng = np.random.default_rng(d + off)
+    tdt, flag = (torch.float32, Z.ZNCC_F32) if dtype == "f32" else (torch.float16, Z.ZNCC_F16)
+    v = rng.integers(-40, 41, (h, w, d)).astype(np.float32)
+    v[0, :, d - 1] = 50.0                                            # the best at either end of a pixel
+    v[1, :, 0] = 50.0
+    v[2, ::2] = -60.0
+    buf = torch.full((16 + off + h * w * d + 16,), 99.0, dtype=tdt, device="cuda")
+    cost = buf[16 + off:16 + off + h * w * d].view(h, w, d)
+    cost.copy_(torch.from_numpy(v))
+    disp = torch.empty((h, w), dtype=torch.int16, device="cuda")
+    with Z.ZnccContext(w, h, d, 3) as ctx:
+        ctx.wta_disparity(cost, disp, flag)
+        torch.cuda.synchronize()
+    assert np.array_equal(disp.cpu().numpy(), v.argmax(-1))
